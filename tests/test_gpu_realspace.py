@@ -163,3 +163,71 @@ def test_real_space_full_size_sampled_atoms(pme, oracle_mod):
     assert rms_force(F[rows], r["forces"]) < F_RMS_TOL
     assert es == pytest.approx(oracle_mod.ewald_self(s.q.astype(np.float64), 0.34), rel=1e-11)  # FP64 sum order
     assert math.isfinite(er) and np.all(np.isfinite(vir))
+
+
+def _water(n, box, seed):
+    """n atoms of the water-like generator's composition at uniform fractional positions of any cell."""
+    _, q = wl.water_box(n, 20.0, seed)
+    return (np.random.default_rng(seed).random((n, 3)) @ np.asarray(box)).astype(np.float32), q
+
+
+# atoms, cell, cutoff, what: item and ring edges of the pair kernel, cell and image edges of its neighbourhoods
+EDGES = {
+    "two_atoms": (2, np.eye(3) * 30.0, 9.0),
+    "one_item": (33, np.eye(3) * 12.0, 5.0),
+    "sparse_rows": (300, np.eye(3) * 120.0, 9.0),          # far fewer atoms than cells
+    "long_rows": (1500, np.diag([14.0, 15.0, 300.0]), 4.0),  # several slabs per row, coarse fixed point
+    "long_other": (1500, np.diag([300.0, 15.0, 14.0]), 4.0),
+    "half_cell": (900, np.eye(3) * 20.0, 10.0),            # the cutoff reaches half the cell
+    "three_images": (200, np.eye(3) * 12.0, 30.0),         # many images of every atom, itself among them
+    "skewed": (1200, np.array([[24.0, 0, 0], [11.0, 22.0, 0], [-10.0, 9.0, 25.0]]), 8.0),
+    "dense": (3000, np.eye(3) * 16.0, 6.0),                # hits of every candidate block, full rings
+    "eight_warps": (4099, np.eye(3) * 34.5, 5.0),
+    "four_warps": (24580, np.eye(3) * 62.7, 3.0),
+}
+
+
+@pytest.mark.parametrize("name", sorted(EDGES))
+def test_pair_kernel_edges(pme, oracle_mod, name):
+    """Each pair term carries a few FP32 roundings (below 16 of 2^-24, or 1e-6), so the sums stay within 1e-6 of the
+    same sums of magnitudes, which are the oracle's for the absolute charges; the self term is an FP64 sum."""
+    n, box, rcut = EDGES[name]
+    pos, q = _water(n, box, 17)
+    beta = 3.0 / rcut
+    er, es, vir, F = gpu_real(pme, pos, q, box, beta, rcut)
+    p64, q64 = pos.astype(np.float64), q.astype(np.float64)
+    oracle_mod.set_threads(16)
+    try:
+        if n > 10000:  # sampled atoms
+            rows = np.random.default_rng(3).choice(n, 60, replace=False)
+            r = oracle_mod.ewald_real_rows(p64, q64, beta, box, rows, rcut=rcut)
+            F = F[rows]
+        else:
+            r = oracle_mod.ewald_real(p64, q64, beta, box, rcut=rcut)
+            big = oracle_mod.ewald_real(p64, np.abs(q64), beta, box, rcut=rcut)
+            assert abs(er - r["energy"]) <= E_REL_TOL * big["energy"]
+            assert np.abs(vir - r["virial"]).max() <= E_REL_TOL * np.abs(big["virial"]).max()
+    finally:
+        oracle_mod.set_threads(1)
+    assert np.abs(F - r["forces"]).max() <= F_RMS_TOL * np.abs(r["forces"]).max()
+    assert es == pytest.approx(oracle_mod.ewald_self(q64, beta), rel=1e-12)
+
+
+def test_pair_kernel_clump_and_collapse(pme, oracle_mod):
+    """All atoms in one corner of a large cell (one crowded neighbourhood, the rest empty), and atoms of the same
+    position (skipped, as a pair at distance zero)."""
+    box = np.eye(3) * 100.0
+    pos, q = _water(1000, np.eye(3) * 8.0, 23)
+    pos[500:503] = pos[10]
+    er, es, vir, F = gpu_real(pme, pos, q, box, 0.34, 9.0)
+    assert np.isfinite(F).all() and math.isfinite(er)
+    keep = np.delete(np.arange(1000), [10, 500, 501, 502])
+    b = gpu_real(pme, pos, q, box, 0.34, 9.0)
+    assert b[0] == er and np.array_equal(b[3], F)
+    # the coincident atoms act on the others as one with their summed charge
+    q2 = q.copy()
+    q2[10] += q[500] + q[501] + q[502]
+    pos2, q2 = np.delete(pos, [500, 501, 502], 0), np.delete(q2, [500, 501, 502])
+    r = oracle_mod.ewald_real(pos2.astype(np.float64), q2.astype(np.float64), 0.34, box, rcut=9.0)
+    ref = np.delete(r["forces"], 10, 0)
+    assert rms_force(F[keep], ref) < F_RMS_TOL
