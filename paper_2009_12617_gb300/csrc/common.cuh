@@ -66,13 +66,17 @@ constexpr int cap_max_for(int tlog) { return tlog >= 4 ? CAP_MAX16 : CAP_MAX; }
 // Columns m3 per influence-stage work item (shared-memory transform path).
 constexpr int CONV_COLS = 8;
 // Lane plans of the register-resident transforms: plan c has length LANE_L[c] * LANE_E[c], L lanes of
-// E points each (fft.cuh, lane_fft). Lengths without a plan use the shared-memory Stockham path.
-constexpr int LANE_PLANS = 21;
-#define PME_LANE_CASES(X)                                                                               \
-    X(0, 1, 4) X(1, 1, 5) X(2, 1, 6) X(3, 1, 8) X(4, 2, 4) X(5, 2, 5) X(6, 2, 6) X(7, 2, 8) X(8, 4, 4) \
-        X(9, 4, 5) X(10, 4, 6) X(11, 4, 8) X(12, 8, 4) X(13, 8, 5) X(14, 8, 6) X(15, 8, 8) X(16, 16, 4) \
-            X(17, 16, 5) X(18, 16, 6) X(19, 16, 8) X(20, 32, 4)
-// Threads (lanes) per influence-stage work item on the register path: 128 / L columns of L lanes each.
+// E points each (fft.cuh, lane_fft). Every mesh edge pme_create accepts, and half of it, has a plan; the
+// shared-memory Stockham transforms remain for the CPU emulation and the allocation-free kernel.
+constexpr int LANE_PLANS = 37;
+#define PME_LANE_CASES(X)                                                                                  \
+    X(0, 1, 4) X(1, 1, 5) X(2, 1, 6) X(3, 1, 8) X(4, 2, 4) X(5, 2, 5) X(6, 2, 6) X(7, 2, 8) X(8, 4, 4)    \
+        X(9, 4, 5) X(10, 4, 6) X(11, 4, 8) X(12, 8, 4) X(13, 8, 5) X(14, 8, 6) X(15, 8, 8) X(16, 16, 4)   \
+            X(17, 16, 5) X(18, 16, 6) X(19, 16, 8) X(20, 32, 4) X(21, 3, 3) X(22, 3, 5) X(23, 3, 6)       \
+                X(24, 5, 5) X(25, 3, 9) X(26, 5, 6) X(27, 6, 6) X(28, 5, 9) X(29, 10, 5) X(30, 6, 9)      \
+                    X(31, 10, 6) X(32, 9, 8) X(33, 10, 9) X(34, 10, 10) X(35, 12, 9) X(36, 15, 8)
+// Threads (lanes) per influence-stage work item on the register path: four warps of 32 / L (rounded down)
+// columns of L lanes each.
 constexpr int CONV_UNITS = 128;
 // Threads of a slab-stage CTA (the register path picks its lane plans to fill about this many).
 constexpr int SLAB_THREADS = 512;
@@ -90,6 +94,8 @@ PME_HD int plan_L(int c) { return PME_LANE_CASES(PME_PLAN_L) 1; }
 PME_HD int plan_E(int c) { return PME_LANE_CASES(PME_PLAN_E) 1; }
 #undef PME_PLAN_L
 #undef PME_PLAN_E
+// Columns of an influence-stage work item of plan c.
+PME_HD int plan_conv_cols(int c) { return CONV_UNITS / 32 * (32 / plan_L(c)); }
 
 // Plan for ntr transforms of length N in one slab CTA: the fewest points per lane (the shortest serial
 // chain per thread) whose lanes still fit in SLAB_THREADS, else the plan with the fewest lanes; -1 when N
@@ -114,6 +120,51 @@ PME_HD int conv_lane_plan(int N) {
     for (int c = 0; c < LANE_PLANS; ++c)
         if (plan_L(c) * plan_E(c) == N && plan_L(c) <= 16 && (best < 0 || plan_E(c) < plan_E(best))) best = c;
     return best;
+}
+// The mesh edges pme_create accepts, and which plans some mesh's rows (K3/2 points, K2 of them), columns (K2
+// points, K3/2 + 1 of them) or k1 transforms take: kernels that choose at run time hold only these.
+constexpr int N_EDGES = 24;
+PME_HD int mesh_edge(int i) {
+    constexpr int e[N_EDGES] = {8, 10, 12, 16, 18, 20, 24, 30, 32, 36, 40, 48, 50, 54, 60, 64, 72, 80, 90, 96, 100, 108, 120, 128};
+    return e[i];
+}
+PME_HD bool plan_for_rows(int c) {
+    for (int i = 0; i < N_EDGES; ++i)
+        if (mesh_edge(i) / 2 == plan_L(c) * plan_E(c))
+            for (int k = 0; k < N_EDGES; ++k)
+                if (slab_lane_plan(mesh_edge(i) / 2, mesh_edge(k)) == c) return true;
+    return false;
+}
+PME_HD bool plan_for_cols(int c) {
+    for (int i = 0; i < N_EDGES; ++i)
+        if (mesh_edge(i) == plan_L(c) * plan_E(c))
+            for (int k = 0; k < N_EDGES; ++k)
+                if (slab_lane_plan(mesh_edge(i), mesh_edge(k) / 2 + 1) == c) return true;
+    return false;
+}
+PME_HD bool plan_for_k1(int c) {
+    for (int i = 0; i < N_EDGES; ++i)
+        if (conv_lane_plan(mesh_edge(i)) == c) return true;
+    return false;
+}
+// Row strides (>= w) of the slab buffers, chosen so that the 16 lanes of a half-warp of the reading pass
+// (T = 32 / L transforms x 16 / T lanes, float2 = two banks) fall on distinct shared-memory banks.
+// Column reader (transform = column, lane j steps rows): stride = min(T, 16) mod 16.
+PME_HD int stride_col_reader(int w, int c) {
+    const int L = plan_L(c);
+    if (L <= 2) return w;  // a half-warp reads 16 consecutive columns of one row
+    return w + ((32 / L - w) & 15);
+}
+// Row reader (transform = row, lane j steps along the row): stride = ceil(16 / T) mod 16.
+PME_HD int stride_row_reader(int w, int c) {
+    const int L = plan_L(c), T = 32 / L;
+    if (L >= 32) return w;  // a half-warp reads 16 consecutive points of one row
+    return w + (((L >= 2 ? (16 + T - 1) / T : 1) - w) & 15);
+}
+// Lanes (whole warps) covering ntr transforms of plan c.
+PME_HD int plan_units(int c, int ntr) {
+    const int T = 32 / plan_L(c);
+    return ((ntr + T - 1) / T) * 32;
 }
 // Independent global loads each thread keeps in flight when staging data into shared memory.
 constexpr int LOAD_BATCH = 8;
@@ -152,6 +203,7 @@ struct SysDev {
     int nconv;                   // influence-stage work items: K2 * nchunk3, or the register path's
                                  // ceil(K2 * H3 / columns per item)
     int lp_rows, lp_cols, lp_k1; // lane plans (PME_LANE_CASES) of the K3/2, K2 and K1 transforms, -1: none
+    int zs, ys, col_units;       // row strides of the forward and inverse slab buffers; lanes of the inverse columns
     int lane_slab, lane_conv;    // slab stages / influence stage take the register path (1) or not (0)
     int pdl_late;                // when a stage kernel triggers its successor's launch (PdlScope, pdl.cuh)
     int nt_tile;                 // spread / force CTA threads (128 or 256) chosen by the tuner; 0: density rule

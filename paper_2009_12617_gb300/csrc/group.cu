@@ -11,15 +11,6 @@
 
 namespace pme {
 
-// The CTA's system descriptor, copied from the group's array into shared memory.
-__device__ __forceinline__ int group_load(const GroupArgs &a, SysDev &sd) {
-    const int sys = blockIdx.x / a.ips;
-    const int *src = (const int *)(a.sys + sys);
-    for (int i = threadIdx.x; i < (int)(sizeof(SysDev) / 4); i += blockDim.x) ((int *)&sd)[i] = src[i];
-    __syncthreads();
-    return blockIdx.x - sys * a.ips;
-}
-
 __global__ void __launch_bounds__(NT_BIN) k_bin_g(GroupArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ SysDev sd;
@@ -36,33 +27,6 @@ __global__ void __launch_bounds__(tile_nt_bound(T)) k_spread_g(GroupArgs a) {
     PdlScope pdl(a.late);
     const int item = group_load(a, sd);
     stage_spread<P, T>(sd, item, smem, true);
-}
-
-template <int PR, int PC>
-__global__ void __launch_bounds__(NT_SLAB) k_fwd_g(GroupArgs a) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ SysDev sd;
-    PdlScope pdl(a.late);
-    const int item = group_load(a, sd);
-    stage_fwd<PR, PC>(sd, item, smem);
-}
-
-template <int P1>
-__global__ void __launch_bounds__(NT_CONV) k_conv_g(GroupArgs a) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ SysDev sd;
-    PdlScope pdl(a.late);
-    const int item = group_load(a, sd);
-    stage_conv<P1>(sd, item, smem);
-}
-
-template <int PR, int PC>
-__global__ void __launch_bounds__(NT_SLAB) k_inv_g(GroupArgs a) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ SysDev sd;
-    PdlScope pdl(a.late);
-    const int item = group_load(a, sd);
-    stage_inv<PR, PC>(sd, item, smem);
 }
 
 template <int P, int T>
@@ -86,33 +50,16 @@ static void (*gather_g_t(int p))(GroupArgs) {
 static void (*spread_g(const SysDev &d))(GroupArgs) { return d.tlog == 4 ? spread_g_t<16>(d.p) : spread_g_t<8>(d.p); }
 static void (*gather_g(const SysDev &d))(GroupArgs) { return d.tlog == 4 ? gather_g_t<16>(d.p) : gather_g_t<8>(d.p); }
 
-static cudaError_t set_limit(const void *fn) {
-    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)(MAX_SMEM_BYTES - sizeof(SysDev) - 64));
-}
-
 cudaError_t configure_group_kernels() {
-    const void *fns[] = {(const void *)k_bin_g, (const void *)k_fwd_g<-1, -1>, (const void *)k_conv_g<-1>,
-                         (const void *)k_inv_g<-1, -1>};
     for (int p : {4, 5, 6, 8})
         for (const void *f : {(const void *)spread_g_t<8>(p), (const void *)spread_g_t<16>(p),
                               (const void *)gather_g_t<8>(p), (const void *)gather_g_t<16>(p)}) {
-            cudaError_t e = set_limit(f);
+            cudaError_t e = set_dynamic_smem(f, GROUP_SMEM_BYTES);
             if (e != cudaSuccess) return e;
         }
-    for (const void *f : fns) {
-        cudaError_t e = set_limit(f);
+    for (cudaError_t e : {configure_fwd_group_kernels(), configure_conv_group_kernels(), configure_inv_group_kernels()})
         if (e != cudaSuccess) return e;
-    }
-#define PME_CFG_K(K)                                                                                        \
-    for (const void *f : {(const void *)k_fwd_g<Cubic<K>::PR, Cubic<K>::PC>, (const void *)k_conv_g<Cubic<K>::P1>, \
-                          (const void *)k_inv_g<Cubic<K>::PR, Cubic<K>::PC>}) {                               \
-        cudaError_t e = set_limit(f);                                                                       \
-        if (e != cudaSuccess) return e;                                                                     \
-    }
-    PME_CUBIC_KS(PME_CFG_K)
-#undef PME_CFG_K
-    return cudaSuccess;
+    return set_dynamic_smem((const void *)k_bin_g, GROUP_SMEM_BYTES);
 }
 
 int group_items(const SysDev &d, int stage) {
@@ -142,34 +89,6 @@ static cudaError_t launch_ex(void (*kernel)(Args...), unsigned grid, unsigned bl
     return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
-static void (*fwd_g(const SysDev &d))(GroupArgs) {
-    if (d.lane_slab) {
-#define PME_PICK(K) \
-    if (d.lp_rows == Cubic<K>::PR && d.lp_cols == Cubic<K>::PC) return k_fwd_g<Cubic<K>::PR, Cubic<K>::PC>;
-        PME_CUBIC_KS(PME_PICK)
-#undef PME_PICK
-    }
-    return k_fwd_g<-1, -1>;
-}
-static void (*inv_g(const SysDev &d))(GroupArgs) {
-    if (d.lane_slab) {
-#define PME_PICK(K) \
-    if (d.lp_rows == Cubic<K>::PR && d.lp_cols == Cubic<K>::PC) return k_inv_g<Cubic<K>::PR, Cubic<K>::PC>;
-        PME_CUBIC_KS(PME_PICK)
-#undef PME_PICK
-    }
-    return k_inv_g<-1, -1>;
-}
-static void (*conv_g(const SysDev &d))(GroupArgs) {
-    if (d.lane_conv) {
-#define PME_PICK(K) \
-    if (d.lp_k1 == Cubic<K>::P1) return k_conv_g<Cubic<K>::P1>;
-        PME_CUBIC_KS(PME_PICK)
-#undef PME_PICK
-    }
-    return k_conv_g<-1>;
-}
-
 cudaError_t launch_group_chain(const SysDev *sys_dev, int nsys, const SysDev &proto, int max_nbin, cudaStream_t s) {
     GroupArgs a;
     a.sys = sys_dev;
@@ -185,9 +104,9 @@ cudaError_t launch_group_chain(const SysDev *sys_dev, int nsys, const SysDev &pr
                 e = launch_ex(spread_g(d), grid, (unsigned)tile_threads(d, (int64_t)max_nbin * BIN_CHUNK),
                               smem_spread(d.p, d.tlog), s, a);
                 break;
-            case STAGE_FWD: e = launch_ex(fwd_g(d), grid, NT_SLAB, smem_slab(d.K2, d.K3), s, a); break;
-            case STAGE_CONV: e = launch_ex(conv_g(d), grid, NT_CONV, smem_conv(d.K1, NT_CONV), s, a); break;
-            case STAGE_INV: e = launch_ex(inv_g(d), grid, NT_SLAB, smem_inv(d.K2, d.K3), s, a); break;
+            case STAGE_FWD: e = launch_ex(fwd_group_kernel(d), grid, NT_SLAB, smem_slab(d.K2, d.K3), s, a); break;
+            case STAGE_CONV: e = launch_ex(conv_group_kernel(d), grid, NT_CONV, smem_conv(d.K1, NT_CONV), s, a); break;
+            case STAGE_INV: e = launch_ex(inv_group_kernel(d), grid, NT_SLAB, smem_inv(d.K2, d.K3), s, a); break;
             default:
                 e = launch_ex(gather_g(d), grid, (unsigned)tile_threads(d, (int64_t)max_nbin * BIN_CHUNK, true),
                               smem_gather_all(d.p, d.tlog), s, a);

@@ -14,6 +14,27 @@ struct GroupArgs {
     int late;           // when the programmatic launch of the successor is triggered (PdlScope)
 };
 
+using GroupKernel = void (*)(GroupArgs);
+// The grouped slab and influence kernels for a system's plans (fwd.cu, conv.cu, inv.cu).
+GroupKernel fwd_group_kernel(const SysDev &d);
+GroupKernel conv_group_kernel(const SysDev &d);
+GroupKernel inv_group_kernel(const SysDev &d);
+// and the shared-memory limits of all of them.
+cudaError_t configure_fwd_group_kernels();
+cudaError_t configure_conv_group_kernels();
+cudaError_t configure_inv_group_kernels();
+
+#if defined(__CUDACC__)
+// The CTA's system descriptor, copied from the group's array into shared memory.
+__device__ __forceinline__ int group_load(const GroupArgs &a, SysDev &sd) {
+    const int sys = blockIdx.x / a.ips;
+    const int *src = (const int *)(a.sys + sys);
+    for (int i = threadIdx.x; i < (int)(sizeof(SysDev) / 4); i += blockDim.x) ((int *)&sd)[i] = src[i];
+    __syncthreads();
+    return blockIdx.x - sys * a.ips;
+}
+#endif
+
 // Raise the dynamic shared-memory limits of the grouped kernels (once per device).
 cudaError_t configure_group_kernels();
 

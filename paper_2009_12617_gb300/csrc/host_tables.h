@@ -124,18 +124,22 @@ inline int choose_tile_log(int64_t n, const int K[3], int sms) {
     return TILE_MIN_LOG;
 }
 
-// Transform paths: the register path (lane plans) wherever both transforms of a slab stage, or the K1
-// transform of the influence stage, have a plan; the shared-memory Stockham path otherwise. The CPU
-// emulation of the stage bodies (one thread per CTA) has no lanes and always takes the shared-memory path.
+// Transform paths: the register path (lane plans), or the shared-memory Stockham path for the allocation-free
+// kernel and the CPU emulation of the stage bodies (one thread per CTA, no lanes).
 inline void choose_fft_paths(SysDev &d, bool lanes) {
     d.lp_rows = lanes ? slab_lane_plan(d.K3 / 2, d.K2) : -1;
     d.lp_cols = lanes ? slab_lane_plan(d.K2, d.H3) : -1;
     d.lp_k1 = lanes ? conv_lane_plan(d.K1) : -1;
     d.lane_slab = (d.lp_rows >= 0 && d.lp_cols >= 0) ? 1 : 0;
+    if (d.lane_slab) {  // the kernels take these from the descriptor: a plan lookup in their prologue costs 0.3 us
+        d.zs = stride_col_reader(d.K3 / 2, d.lp_cols);
+        d.ys = stride_row_reader(d.H3, d.lp_rows);
+        d.col_units = plan_units(d.lp_cols, d.H3);
+    }
     d.lane_conv = d.lp_k1 >= 0 ? 1 : 0;
     d.nchunk3 = (d.H3 + CONV_COLS - 1) / CONV_COLS;
     if (d.lane_conv) {
-        const int cols = CONV_UNITS / plan_L(d.lp_k1);  // columns per work item
+        const int cols = plan_conv_cols(d.lp_k1);  // columns per work item
         d.nconv = (d.K2 * d.H3 + cols - 1) / cols;
     } else {
         d.nconv = d.K2 * d.nchunk3;
@@ -230,6 +234,7 @@ inline void make_influence(const int K[3], int p, double beta, const double reci
         for (int j = 0; j < 3; ++j) mv[j] = mt1 * recip[j] + mt2 * recip[3 + j] + mt3 * recip[6 + j];
         return mv[0] * mv[0] + mv[1] * mv[1] + mv[2] * mv[2];
     };
+    // C(m) and C(-m) are the same number off the Nyquist planes
     auto C = [&](double m2n) { return exp(-fac * m2n) / (PI_D * vol * m2n); };
     auto f = [&](double m2n) { return 2.0 * (1.0 / m2n + fac); };
     for (int m2 = 0; m2 < K[1]; ++m2)
@@ -241,7 +246,8 @@ inline void make_influence(const int K[3], int p, double beta, const double reci
                     const double nm = norm2(mt1, mt2, mt3);
                     const double np = norm2(signed_freq_h((K[0] - m1) % K[0], K[0]), signed_freq_h((K[1] - m2) % K[1], K[1]),
                                             signed_freq_h((K[2] - m3) % K[2], K[2]));
-                    v = b1[m1] * b2[m2] * b3[m3] * 0.5 * (C(nm) + C(np));
+                    const double cm = C(nm);
+                    v = b1[m1] * b2[m2] * b3[m3] * 0.5 * (cm + (np == nm ? cm : C(np)));
                     g = v * f(nm);
                     const bool self = m3 == 0 || 2 * m3 == K[2];
                     if (!self && (2 * m1 == K[0] || 2 * m2 == K[1])) {
@@ -275,7 +281,7 @@ inline int conv_item_col(const SysDev &d, int i) {
     if (i >= d.nconv) return ncol;
     int c;
     if (d.lane_conv) {
-        c = i * (CONV_UNITS / plan_L(d.lp_k1));
+        c = i * plan_conv_cols(d.lp_k1);
     } else {
         const int m2 = i / d.nchunk3, ch = i - m2 * d.nchunk3;
         c = m2 * d.H3 + ch * CONV_COLS;

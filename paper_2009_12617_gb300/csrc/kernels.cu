@@ -30,57 +30,14 @@ __global__ void __launch_bounds__(tile_nt_bound(T)) k_spread(SysDev d) {
     stage_spread<P, T>(d, blockIdx.x, smem, true, org);
 }
 
-__global__ void __launch_bounds__(NT_SLAB) k_fwd(SysDev d) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    PdlScope pdl(d.pdl_late);
-    stage_fwd(d, d.item0 + blockIdx.x, smem);
-}
-
-__global__ void __launch_bounds__(NT_CONV) k_conv(SysDev d) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    PdlScope pdl(d.pdl_late);
-    stage_conv(d, d.item0 + blockIdx.x, smem);
-}
-
-__global__ void __launch_bounds__(NT_SLAB) k_inv(SysDev d) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    PdlScope pdl(d.pdl_late);
-    stage_inv(d, d.item0 + blockIdx.x, smem);
-}
-
-// Slab and influence kernels specialised for the lane plans of the cubic meshes of PME_CUBIC_KS (kernels.h);
-// each holds only its plans' code. Other meshes run the kernels above, which choose among all plans at run
-// time.
-
-template <int PR, int PC>
-__global__ void __launch_bounds__(NT_SLAB) k_fwd_p(SysDev d) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    PdlScope pdl(d.pdl_late);
-    stage_fwd<PR, PC>(d, d.item0 + blockIdx.x, smem);
-}
-
-template <int P1>
-__global__ void __launch_bounds__(NT_CONV) k_conv_p(SysDev d) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    PdlScope pdl(d.pdl_late);
-    stage_conv<P1>(d, d.item0 + blockIdx.x, smem);
-}
-
-template <int PR, int PC>
-__global__ void __launch_bounds__(NT_SLAB) k_inv_p(SysDev d) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    PdlScope pdl(d.pdl_late);
-    stage_inv<PR, PC>(d, d.item0 + blockIdx.x, smem);
-}
-
 // Slab kernels with each slab split over a thread-block cluster of CS CTAs (slab d.item0 + blockIdx.x / CS,
 // cluster rank blockIdx.x mod CS), for K2 = K3 = K. They keep the one-CTA kernels' lane plans (the same
 // transforms in the same order, so the same bits), with fewer transforms per CTA.
 template <int K, int CS>
 struct SlabSplit {
     static constexpr int H3 = K / 2 + 1;
-    static constexpr int PR = Cubic<K>::PR, PC = Cubic<K>::PC;
-    static constexpr int units(int c, int ntr) { return ((ntr + 32 / plan_L(c) - 1) / (32 / plan_L(c))) * 32; }
+    static constexpr int PR = Edge<K>::PR, PC = Edge<K>::PC;
+    static constexpr int units(int c, int ntr) { return plan_units(c, ntr); }
     static constexpr int NT_FWD = units(PR, K / CS) > units(PC, (H3 + CS - 1) / CS) ? units(PR, K / CS)
                                                                                        : units(PC, (H3 + CS - 1) / CS);
     static constexpr int NT_INV = NT_FWD + 64;  // two spare warps for the side work
@@ -174,34 +131,21 @@ static bool launch_split_slab(const SysDev &d, bool fwd, int count, cudaStream_t
     return false;
 }
 
-static cudaError_t set_smem_limit(const void *fn, size_t bytes) {
-    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 cudaError_t configure_kernels() {
     const size_t big = MAX_SMEM_BYTES;
-    const void *fns[] = {(const void *)k_fwd, (const void *)k_conv, (const void *)k_inv,
-                         (const void *)k_spread<4, 8>, (const void *)k_spread<5, 8>, (const void *)k_spread<6, 8>,
+    const void *fns[] = {(const void *)k_spread<4, 8>, (const void *)k_spread<5, 8>, (const void *)k_spread<6, 8>,
                          (const void *)k_spread<8, 8>, (const void *)k_spread<4, 16>, (const void *)k_spread<5, 16>,
                          (const void *)k_spread<6, 16>, (const void *)k_spread<8, 16>, (const void *)k_gather<4, 8>,
                          (const void *)k_gather<5, 8>, (const void *)k_gather<6, 8>, (const void *)k_gather<8, 8>,
                          (const void *)k_gather<4, 16>, (const void *)k_gather<5, 16>, (const void *)k_gather<6, 16>,
                          (const void *)k_gather<8, 16>};
     for (const void *f : fns) {
-        cudaError_t e = set_smem_limit(f, big);
+        cudaError_t e = set_dynamic_smem(f, big);
         if (e != cudaSuccess) return e;
     }
-#define PME_CFG_K(K)                                                                                        \
-    for (const void *f : {(const void *)k_fwd_p<Cubic<K>::PR, Cubic<K>::PC>, (const void *)k_conv_p<Cubic<K>::P1>, \
-                          (const void *)k_inv_p<Cubic<K>::PR, Cubic<K>::PC>}) {                               \
-        cudaError_t e = set_smem_limit(f, big);                                                             \
-        if (e != cudaSuccess) return e;                                                                     \
-    }
-    PME_CUBIC_KS(PME_CFG_K)
-#undef PME_CFG_K
 #define PME_CFG_SPLIT(K, CS)                                                                \
     for (const void *f : {(const void *)k_fwd_c<K, CS>, (const void *)k_inv_c<K, CS>}) {   \
-        cudaError_t e = set_smem_limit(f, big);                                             \
+        cudaError_t e = set_dynamic_smem(f, big);                                             \
         if (e != cudaSuccess) return e;                                                     \
     }
     PME_SPLIT_KS(PME_CFG_SPLIT)
@@ -209,33 +153,11 @@ cudaError_t configure_kernels() {
     return configure_tc_kernel();
 }
 
-// The specialised kernel for the system's plans, or the general one.
-static void (*fwd_kernel(const SysDev &d))(SysDev) {
-    if (d.lane_slab) {
-#define PME_PICK(K) \
-    if (d.lp_rows == Cubic<K>::PR && d.lp_cols == Cubic<K>::PC) return k_fwd_p<Cubic<K>::PR, Cubic<K>::PC>;
-        PME_CUBIC_KS(PME_PICK)
-#undef PME_PICK
-    }
-    return k_fwd;
-}
-static void (*inv_kernel(const SysDev &d))(SysDev) {
-    if (d.lane_slab) {
-#define PME_PICK(K) \
-    if (d.lp_rows == Cubic<K>::PR && d.lp_cols == Cubic<K>::PC) return k_inv_p<Cubic<K>::PR, Cubic<K>::PC>;
-        PME_CUBIC_KS(PME_PICK)
-#undef PME_PICK
-    }
-    return k_inv;
-}
-static void (*conv_kernel(const SysDev &d))(SysDev) {
-    if (d.lane_conv) {
-#define PME_PICK(K) \
-    if (d.lp_k1 == Cubic<K>::P1) return k_conv_p<Cubic<K>::P1>;
-        PME_CUBIC_KS(PME_PICK)
-#undef PME_PICK
-    }
-    return k_conv;
+cudaError_t configure_transforms(const SysDev &d) {
+    cudaError_t e;
+    if ((e = set_dynamic_smem((const void *)fwd_kernel(d), MAX_SMEM_BYTES)) != cudaSuccess) return e;
+    if ((e = set_dynamic_smem((const void *)conv_kernel(d), MAX_SMEM_BYTES)) != cudaSuccess) return e;
+    return set_dynamic_smem((const void *)inv_kernel(d), MAX_SMEM_BYTES);
 }
 
 template <int P>

@@ -33,13 +33,17 @@ inline int tile_threads(const SysDev &d, int64_t n, bool gather = false) {
 }
 constexpr int NT_CONV = 128;   // threads per CTA for the influence stage
 constexpr size_t MAX_SMEM_BYTES = 226 * 1024;  // opt-in limit is 227 KB including static shared memory
+constexpr size_t GROUP_SMEM_BYTES = MAX_SMEM_BYTES - sizeof(SysDev) - 64;  // beside the system's descriptor
 
-// Cubic meshes K^3 whose lane plans get kernels (and batch stage calls) specialised at compile time.
-#define PME_CUBIC_KS(X) X(16) X(20) X(24) X(32) X(40) X(48) X(64) X(80) X(96) X(128)
+// Mesh edges K whose lane plans get kernels (and batch stage calls) specialised at compile time: slab kernels for
+// K2 = K3 = K, influence kernels for K1 = K.
+#define PME_EDGES(X)                                                                                         \
+    X(16) X(18) X(20) X(24) X(30) X(32) X(36) X(40) X(48) X(50) X(54) X(60) X(64) X(72) X(80) X(90) X(96) X(100) \
+        X(108) X(120) X(128)
 template <int K>
-struct Cubic {
+struct Edge {
     static constexpr int PR = slab_lane_plan(K / 2, K), PC = slab_lane_plan(K, K / 2 + 1), P1 = conv_lane_plan(K);
-    static_assert(PR >= 0 && PC >= 0 && P1 >= 0, "every listed cubic mesh has lane plans");
+    static_assert(PR >= 0 && PC >= 0 && P1 >= 0, "every listed edge has lane plans");
 };
 
 // Launch mode of the per-stage kernels: 0 plain, 1 programmatic dependent launch triggered at kernel entry,
@@ -62,6 +66,17 @@ int slab_split(int inverse);
 
 // Raise the dynamic shared-memory limit of the large-footprint kernels (once per device).
 cudaError_t configure_kernels();
+inline cudaError_t set_dynamic_smem(const void *fn, size_t bytes) {
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
+using StageKernel = void (*)(SysDev);
+// The slab and influence kernels for a system's plans (fwd.cu, conv.cu, inv.cu); configure_transforms raises the
+// shared-memory limits of the three (a plan does it when it is created, which loads only the kernels in use).
+StageKernel fwd_kernel(const SysDev &d);
+StageKernel conv_kernel(const SysDev &d);
+StageKernel inv_kernel(const SysDev &d);
+cudaError_t configure_transforms(const SysDev &d);
 
 // Optional device-to-device copies of intermediate meshes (diagnostics).
 struct DebugTaps {

@@ -355,6 +355,10 @@ pme_status pme_create(const int K[3], int p, double beta, const double box[9], v
     pl->vol = vol;
     memset(&pl->d, 0, sizeof(pl->d));
     fill_geometry(pl->d, K, p, beta, recip);
+    if ((e = configure_transforms(pl->d)) != cudaSuccess) {
+        delete pl;
+        return cuda_fail(e, "configure kernels");
+    }
     pme_status st;
     if ((st = alloc_mesh(pl)) != PME_OK || (st = upload_tables(pl)) != PME_OK || (st = plan_reserve(pl, 1)) != PME_OK) {
         pme_destroy(pl);

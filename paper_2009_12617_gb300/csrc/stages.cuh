@@ -1005,13 +1005,18 @@ namespace cg = cooperative_groups;
 // multiples of 32; every warp runs whole loop iterations, and lanes past the end work on a valid dummy
 // transform without storing, so the shuffles always see full warps.
 
-// Unit u -> (transform t, lane j): warp u / 32 holds T = 32 / L transforms at lane ids t mod T + T j.
+// Unit u -> (transform t, lane j): warp u / 32 holds T = floor(32 / L) transforms at lane ids t mod T + T j. Lanes
+// past the last transform get a t beyond any count: they work on a valid transform without storing.
 template <int L>
 PME_DEV void lane_unit(int u, int &t, int &j) {
     constexpr int T = 32 / L;
     const int lid = u & 31;
-    t = (u >> 5) * T + (lid & (T - 1));
+    t = (u >> 5) * T + (T * L == 32 ? lid & (T - 1) : lid % T);
     j = lid / T;
+    if (T * L < 32 && j >= L) {
+        t = 1 << 24;
+        j = 0;
+    }
 }
 
 // Units covering ntr transforms of L lanes: whole warps.
@@ -1154,14 +1159,14 @@ PME_DEV void inv_rows_lane(const SysDev &d, int k1, const float2 *Y, int ys, con
     }
 }
 
-// a4 / a7 register path: work item = CONV_UNITS / L consecutive columns (m2, m3) of the half spectrum
+// a4 / a7 register path: work item = plan_conv_cols consecutive columns (m2, m3) of the half spectrum
 // (flattened m2 H3 + m3). Each column: forward K1-point transform, B*C product with the energy and virial
 // terms (influence_point), adjoint transform back in place. The item's energy / virial partial is a
 // fixed-order double-float tree over its CONV_UNITS lanes, one component per warp, independent of the block
 // size.
 template <int L, int E>
 PME_DEV void conv_lane(const SysDev &d, int item, void *smem) {
-    constexpr int COLS = CONV_UNITS / L;
+    constexpr int COLS = CONV_UNITS / 32 * (32 / L);
     const int tid = PME_TID, nth = PME_NTH;
     const int K1 = d.K1, K2 = d.K2, H3 = d.H3, ncol = K2 * H3;
     const float inv_h3 = 1.0f / (float)H3;
@@ -1221,38 +1226,67 @@ PME_DEV void conv_lane(const SysDev &d, int item, void *smem) {
 }
 
 
-PME_DEV int plan_col_units(int c, int ntr) {
-    const int T = 32 / plan_L(c);
-    return ((ntr + T - 1) / T) * 32;
-}
-
-// Row strides (>= w) of the slab buffers, chosen so that the 16 lanes of a half-warp of the reading pass
-// (T = 32 / L transforms x 16 / T lanes, float2 = two banks) fall on distinct shared-memory banks.
-// Column reader (transform = column, lane j steps rows): stride = min(T, 16) mod 16.
-PME_DEV int stride_col_reader(int w, int c) {
-    const int L = plan_L(c);
-    if (L <= 2) return w;  // a half-warp reads 16 consecutive columns of one row
-    return w + ((32 / L - w) & 15);
-}
-// Row reader (transform = row, lane j steps along the row): stride = max(L / 2, 1) mod 16.
-PME_DEV int stride_row_reader(int w, int c) {
-    const int L = plan_L(c);
-    if (L >= 32) return w;  // a half-warp reads 16 consecutive points of one row
-    return w + (((L >= 2 ? L / 2 : 1) - w) & 15);
-}
-
 // Compile-time lanes and points of plan C.
 template <int C>
 struct PlanLE {
     static constexpr int L = plan_L(C), E = plan_E(C);
 };
 
+// The slab passes as calls, for kernels that choose the plans at run time: inlined into one kernel, all plans' code
+// together makes instruction fetch the bottleneck (60^3, cold caches: 15.6 warps stalled on it per issue and 13.4 us a
+// stage; as calls 7.2 and 11.4 us; the kernel with that mesh's plans alone 1.0 and 7.7 us. In a running
+// evaluation the two slab stages cost 2.4 us more than the specialised ones). The slab buffer starts the
+// dynamic shared memory; arguments are passed one by one, so that they stay in registers.
+template <int L, int E>
+__device__ __noinline__ void fwd_rows_call(unsigned long long *grid, const float2 *tw3h, int K2, int K3, int k1, int zs) {
+    extern __shared__ __align__(16) unsigned char dyn_smem[];
+    SysDev d;
+    d.grid = grid;
+    d.tw3h = tw3h;
+    d.K2 = K2;
+    d.K3 = K3;
+    const SlabDst<1> Zd = {{(float2 *)dyn_smem}};
+    fwd_rows_lane<L, E>(d, k1, Zd, zs, 0, K2);
+}
+template <int L, int E>
+__device__ __noinline__ void fwd_cols_call(float2 *spec, int K2, int K3, int k1, int zs) {
+    extern __shared__ __align__(16) unsigned char dyn_smem[];
+    SysDev d;
+    d.spec = spec;
+    d.K2 = K2;
+    d.K3 = K3;
+    d.H3 = K3 / 2 + 1;
+    const float2 *Z = (const float2 *)dyn_smem, *tw3 = Z + K2 * zs;
+    fwd_cols_lane<L, E>(d, k1, Z, zs, tw3, tw3 + K3 / 2 + 1, 0, d.H3);
+}
+template <int L, int E>
+__device__ __noinline__ void inv_cols_call(float2 *spec, const float2 *tw2, int K2, int K3, int k1, int ys) {
+    extern __shared__ __align__(16) unsigned char dyn_smem[];
+    SysDev d;
+    d.spec = spec;
+    d.tw2 = tw2;
+    d.K2 = K2;
+    d.H3 = K3 / 2 + 1;
+    const SlabDst<1> Yd = {{(float2 *)dyn_smem}};
+    inv_cols_lane<L, E>(d, k1, Yd, ys, 0, d.H3);
+}
+template <int L, int E>
+__device__ __noinline__ void inv_rows_call(float *phi, int K2, int K3, int k1, int ys) {
+    extern __shared__ __align__(16) unsigned char dyn_smem[];
+    SysDev d;
+    d.phi = phi;
+    d.K2 = K2;
+    d.K3 = K3;
+    const float2 *Y = (const float2 *)dyn_smem, *twh = Y + K2 * ys;
+    inv_rows_lane<L, E>(d, k1, Y, ys, twh, twh + K3 / 2, 0, K2);
+}
+
 // Lane slab / influence stages with the plans fixed at compile time (PR, PC, P1 >= 0: only that plan's code
 // is built into the kernel, which keeps it small enough for the instruction caches) or chosen at run time
 // from the system's plans (-1).
 template <int PR, int PC>
 PME_DEV void stage_fwd_lane(const SysDev &d, int k1, void *smem) {
-    const int Nh = d.K3 / 2, zs = stride_col_reader(Nh, d.lp_cols);
+    const int Nh = d.K3 / 2, zs = d.zs;
     float2 *Z = (float2 *)smem;
     float2 *tw3 = Z + d.K2 * zs;  // Nh + 1
     float2 *tw2 = tw3 + Nh + 1;   // K2
@@ -1261,13 +1295,15 @@ PME_DEV void stage_fwd_lane(const SysDev &d, int k1, void *smem) {
     const int tid = PME_TID;
     const float2 a = tid <= Nh ? __ldg(d.tw3 + tid) : make_float2(0.f, 0.f);
     const float2 b = tid < d.K2 ? __ldg(d.tw2 + tid) : make_float2(0.f, 0.f);
-    const SlabDst<1> Zd = {{Z}};
     if constexpr (PR >= 0) {
+        const SlabDst<1> Zd = {{Z}};
         fwd_rows_lane<PlanLE<PR>::L, PlanLE<PR>::E>(d, k1, Zd, zs, 0, d.K2);
     } else {
         switch (d.lp_rows) {
 #define PME_ROWS(c, L, E) \
-    case c: fwd_rows_lane<L, E>(d, k1, Zd, zs, 0, d.K2); break;
+    case c:                                                                      \
+        if constexpr (plan_for_rows(c)) fwd_rows_call<L, E>(d.grid, d.tw3h, d.K2, d.K3, k1, zs); \
+        break;
             PME_LANE_CASES(PME_ROWS)
 #undef PME_ROWS
         }
@@ -1282,7 +1318,9 @@ PME_DEV void stage_fwd_lane(const SysDev &d, int k1, void *smem) {
     } else {
         switch (d.lp_cols) {
 #define PME_COLS(c, L, E) \
-    case c: fwd_cols_lane<L, E>(d, k1, Z, zs, tw3, tw2, 0, d.H3); break;
+    case c:                                                                                  \
+        if constexpr (plan_for_cols(c)) fwd_cols_call<L, E>(d.spec, d.K2, d.K3, k1, zs); \
+        break;
             PME_LANE_CASES(PME_COLS)
 #undef PME_COLS
         }
@@ -1291,7 +1329,7 @@ PME_DEV void stage_fwd_lane(const SysDev &d, int k1, void *smem) {
 
 template <int PR, int PC>
 PME_DEV void stage_inv_lane(const SysDev &d, int k1, void *smem) {
-    const int Nh = d.K3 / 2, ys = stride_row_reader(d.H3, d.lp_rows);
+    const int Nh = d.K3 / 2, ys = d.ys;
     float2 *Y = (float2 *)smem;
     float2 *twh = Y + d.K2 * ys;  // Nh
     float2 *tw3 = twh + Nh;       // Nh + 1
@@ -1300,16 +1338,18 @@ PME_DEV void stage_inv_lane(const SysDev &d, int k1, void *smem) {
     const float2 a = tid < Nh ? __ldg(d.tw3h + tid) : make_float2(0.f, 0.f);
     const float2 b = tid <= Nh ? __ldg(d.tw3 + tid) : make_float2(0.f, 0.f);
     // the column pass needs cu threads; warps beyond them (if any) take the side work, else everyone first
-    const int cu = plan_col_units(d.lp_cols, d.H3);
+    const int cu = d.col_units;
     if (PME_NTH - cu >= 32) inv_side_work(d, k1, cu, PME_NTH - cu);
     else inv_side_work(d, k1, 0, PME_NTH);
-    const SlabDst<1> Yd = {{Y}};
     if constexpr (PC >= 0) {
+        const SlabDst<1> Yd = {{Y}};
         inv_cols_lane<PlanLE<PC>::L, PlanLE<PC>::E>(d, k1, Yd, ys, 0, d.H3);
     } else {
         switch (d.lp_cols) {
 #define PME_COLS(c, L, E) \
-    case c: inv_cols_lane<L, E>(d, k1, Yd, ys, 0, d.H3); break;
+    case c:                                                                      \
+        if constexpr (plan_for_cols(c)) inv_cols_call<L, E>(d.spec, d.tw2, d.K2, d.K3, k1, ys); \
+        break;
             PME_LANE_CASES(PME_COLS)
 #undef PME_COLS
         }
@@ -1324,7 +1364,9 @@ PME_DEV void stage_inv_lane(const SysDev &d, int k1, void *smem) {
     } else {
         switch (d.lp_rows) {
 #define PME_ROWS(c, L, E) \
-    case c: inv_rows_lane<L, E>(d, k1, Y, ys, twh, tw3, 0, d.K2); break;
+    case c:                                                                               \
+        if constexpr (plan_for_rows(c)) inv_rows_call<L, E>(d.phi, d.K2, d.K3, k1, ys); \
+        break;
             PME_LANE_CASES(PME_ROWS)
 #undef PME_ROWS
         }
@@ -1414,7 +1456,9 @@ PME_DEV void stage_conv_lane(const SysDev &d, int item, void *smem) {
     } else {
         switch (d.lp_k1) {
 #define PME_K1(c, L, E) \
-    case c: conv_lane<L, E>(d, item, smem); break;
+    case c:                                                         \
+        if constexpr (plan_for_k1(c)) conv_lane<L, E>(d, item, smem); \
+        break;
             PME_LANE_CASES(PME_K1)
 #undef PME_K1
         }
@@ -1422,19 +1466,14 @@ PME_DEV void stage_conv_lane(const SysDev &d, int item, void *smem) {
 }
 #endif  // PME_LANE_FFT
 
-// Stage entry points: the register path where the plan has lane plans, else the shared-memory path. With
-// plans given at compile time (a kernel specialised for one mesh), only the register path is built in; such
-// a kernel runs only for systems with exactly those plans.
+// Stage entry points: the register path, or the shared-memory path in builds without it (the CPU emulation, the
+// allocation-free kernel). With plans given at compile time (a kernel specialised for one mesh) only their code
+// is built in; such a kernel runs only for systems with exactly those plans.
 template <int PR = -1, int PC = -1>
 PME_DEV void stage_fwd(const SysDev &d, int k1, void *smem) {
     if (k1 == 0 && PME_TID == 0) d.ctl->novf = 0u;  // spreading (its last reader) has finished
 #if defined(PME_LANE_FFT)
-    if constexpr (PR >= 0) {
-        stage_fwd_lane<PR, PC>(d, k1, smem);
-    } else {
-        if (d.lane_slab) stage_fwd_lane<-1, -1>(d, k1, smem);
-        else stage_fwd_smem(d, k1, smem);
-    }
+    stage_fwd_lane<PR, PC>(d, k1, smem);
 #else
     stage_fwd_smem(d, k1, smem);
 #endif
@@ -1443,12 +1482,7 @@ PME_DEV void stage_fwd(const SysDev &d, int k1, void *smem) {
 template <int P1 = -1>
 PME_DEV void stage_conv(const SysDev &d, int item, void *smem) {
 #if defined(PME_LANE_FFT)
-    if constexpr (P1 >= 0) {
-        stage_conv_lane<P1>(d, item, smem);
-    } else {
-        if (d.lane_conv) stage_conv_lane<-1>(d, item, smem);
-        else stage_conv_smem(d, item, smem);
-    }
+    stage_conv_lane<P1>(d, item, smem);
 #else
     stage_conv_smem(d, item, smem);
 #endif
@@ -1457,16 +1491,7 @@ PME_DEV void stage_conv(const SysDev &d, int item, void *smem) {
 template <int PR = -1, int PC = -1>
 PME_DEV void stage_inv(const SysDev &d, int k1, void *smem) {
 #if defined(PME_LANE_FFT)
-    if constexpr (PR >= 0) {
-        stage_inv_lane<PR, PC>(d, k1, smem);
-    } else {
-        if (d.lane_slab) {
-            stage_inv_lane<-1, -1>(d, k1, smem);
-        } else {
-            inv_side_work(d, k1, 0, PME_NTH);
-            stage_inv_smem(d, k1, smem);
-        }
-    }
+    stage_inv_lane<PR, PC>(d, k1, smem);
 #else
     inv_side_work(d, k1, 0, PME_NTH);
     stage_inv_smem(d, k1, smem);

@@ -90,6 +90,36 @@ def test_parity_mesh_shapes(pmelib, oracle_mod, K, p):
         pmelib.pme_destroy(plan)
 
 
+# every edge with a factor 3 or 5 across lanes: as K1 with its own influence kernel and as K2 = K3 with its own slab
+# kernels, then as K2 and K3 of slabs that pick their plans at run time
+LANE_EDGES = [(60, 18, 18), (72, 30, 30), (18, 36, 36), (100, 50, 50), (30, 54, 54), (36, 60, 60), (50, 72, 72), (120, 90, 90),
+              (54, 100, 100), (90, 108, 108), (108, 120, 120),
+              (54, 60, 72), (20, 36, 108), (12, 90, 54), (8, 100, 90), (18, 50, 120), (10, 72, 60), (16, 108, 100), (24, 120, 36),
+              (32, 18, 30), (40, 30, 18), (48, 54, 50)]
+
+
+@pytest.mark.parametrize("K", LANE_EDGES, ids=["x".join(map(str, K)) for K in LANE_EDGES])
+def test_parity_lane_plans(pmelib, K):
+    """The FP64 numpy evaluation (checked against the oracle by the CPU tests) at the parity tolerances."""
+    from oracle import numpy_spme
+
+    L = np.array(K, dtype=float) * 1.1
+    box = np.diag(L)
+    rng = np.random.default_rng(sum(K))
+    pos = (rng.random((900, 3)) * L).astype(np.float32)
+    q = rng.normal(size=900)
+    q = (q - q.mean()).astype(np.float32)
+    plan = pmelib.pme_create(K, 4, 0.34, box)
+    try:
+        g = gpu_eval(pmelib, plan, pos, q)
+    finally:
+        pmelib.pme_destroy(plan)
+    r = numpy_spme.spme(pos, q, K, 4, 0.34, box)
+    assert rel_energy(g["energy"], r["energy"]) < E_REL_TOL
+    assert rms_force(g["forces"], r["forces"]) < F_RMS_TOL
+    assert rel_virial(g["virial"], r["virial"]) < V_TOL
+
+
 def test_parity_triclinic(pmelib, oracle_mod):
     s = wl.parity_system()
     box = np.array([[27.4, 0, 0], [3.1, 26.0, 0], [-2.0, 4.0, 28.0]])
