@@ -220,10 +220,10 @@ void pme_destroy(pme_plan *plan);
  * spectrum, influence table, recomputed on the device every call, bucket lists, counters) lives in one
  * static device array of 4 MiB that every GPU loading the library holds until the process exits.
  * Limits: K1*K2*K3 <= 32768 with each K_alpha <= 64, n <= 16384, and the carved scratch must fit in 4 MiB;
- * anything larger returns PME_EINVAL with the reason. One cooperative kernel launch on cuda_stream, then the
- * call waits for it. The first call on a device looks up the array's device address (cudaGetSymbolAddress)
- * and the cooperative grid size, so make that first call before any stream capture. Every call starts by
- * clearing the parts of the array that must be zero, but all calls share the one array: calls that overlap
+ * anything larger returns PME_EINVAL with the reason. A chain of kernel launches on cuda_stream, then the
+ * call waits for them. The first call on a device looks up the array's device address (cudaGetSymbolAddress),
+ * loads every kernel a later call may launch and sets a page-locked result block aside, so make that first call
+ * before any stream capture. Every call starts by clearing the parts of the array that must be zero, but all calls share the one array: calls that overlap
  * on the GPU (from different streams or threads) race and give wrong results. */
 pme_status pme_compute_noalloc(const int K[3], int p, double beta, const double box[9], const float *pos,
                                const float *q, int64_t n, float *forces, double *energy, double *virial,

@@ -67,7 +67,7 @@ constexpr int cap_max_for(int tlog) { return tlog >= 4 ? CAP_MAX16 : CAP_MAX; }
 constexpr int CONV_COLS = 8;
 // Lane plans of the register-resident transforms: plan c has length LANE_L[c] * LANE_E[c], L lanes of
 // E points each (fft.cuh, lane_fft). Every mesh edge pme_create accepts, and half of it, has a plan; the
-// shared-memory Stockham transforms remain for the CPU emulation and the allocation-free kernel.
+// shared-memory Stockham transforms remain for the CPU emulation.
 constexpr int LANE_PLANS = 37;
 #define PME_LANE_CASES(X)                                                                                  \
     X(0, 1, 4) X(1, 1, 5) X(2, 1, 6) X(3, 1, 8) X(4, 2, 4) X(5, 2, 5) X(6, 2, 6) X(7, 2, 8) X(8, 4, 4)    \
@@ -127,6 +127,11 @@ constexpr int N_EDGES = 24;
 PME_HD int mesh_edge(int i) {
     constexpr int e[N_EDGES] = {8, 10, 12, 16, 18, 20, 24, 30, 32, 36, 40, 48, 50, 54, 60, 64, 72, 80, 90, 96, 100, 108, 120, 128};
     return e[i];
+}
+PME_HD int edge_index(int K) {
+    for (int i = 0; i < N_EDGES; ++i)
+        if (mesh_edge(i) == K) return i;
+    return -1;
 }
 PME_HD bool plan_for_rows(int c) {
     for (int i = 0; i < N_EDGES; ++i)

@@ -124,8 +124,8 @@ inline int choose_tile_log(int64_t n, const int K[3], int sms) {
     return TILE_MIN_LOG;
 }
 
-// Transform paths: the register path (lane plans), or the shared-memory Stockham path for the allocation-free
-// kernel and the CPU emulation of the stage bodies (one thread per CTA, no lanes).
+// Transform paths: the register path (lane plans), or the shared-memory Stockham path for the CPU emulation of the
+// stage bodies (one thread per CTA, no lanes).
 inline void choose_fft_paths(SysDev &d, bool lanes) {
     d.lp_rows = lanes ? slab_lane_plan(d.K3 / 2, d.K2) : -1;
     d.lp_cols = lanes ? slab_lane_plan(d.K2, d.H3) : -1;

@@ -153,6 +153,34 @@ cudaError_t configure_kernels() {
     return configure_tc_kernel();
 }
 
+// Forces from device memory to page-locked host memory (coalesced 16-byte stores where both addresses
+// allow) and the control block to its host copy: the last step of an evaluation on host arrays.
+__global__ void __launch_bounds__(256) k_copy_out(const float *src, float *dst, long long nf, const Ctl *ctl, Ctl *hctl,
+                                                  double *res8) {
+    pdl_wait();
+    const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x, nth = (long long)gridDim.x * blockDim.x;
+    if (((((size_t)src) | ((size_t)dst)) & 15) == 0) {
+        const long long n4 = nf >> 2;
+        for (long long i = tid; i < n4; i += nth) ((float4 *)dst)[i] = __ldcg((const float4 *)src + i);
+        for (long long i = (n4 << 2) + tid; i < nf; i += nth) dst[i] = __ldcg(src + i);
+    } else {
+        for (long long i = tid; i < nf; i += nth) dst[i] = __ldcg(src + i);
+    }
+    if (hctl && blockIdx.x == 0 && threadIdx.x < sizeof(Ctl) / 4)
+        ((unsigned *)hctl)[threadIdx.x] = __ldcg((const unsigned *)ctl + threadIdx.x);
+    if (res8 && blockIdx.x == 0 && threadIdx.x < 8)  // energy, virial[6], status bits
+        res8[threadIdx.x] = threadIdx.x < 7 ? __ldcg(ctl->ev + threadIdx.x) : (double)__ldcg(&ctl->status);
+}
+
+cudaError_t load_stage_kernels() {
+    cudaFuncAttributes a;
+    for (const void *f : {(const void *)k_bin, (const void *)k_copy_out}) {
+        cudaError_t e = cudaFuncGetAttributes(&a, f);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
 cudaError_t configure_transforms(const SysDev &d) {
     cudaError_t e;
     if ((e = set_dynamic_smem((const void *)fwd_kernel(d), MAX_SMEM_BYTES)) != cudaSuccess) return e;
@@ -236,25 +264,6 @@ void launch_stage_items(const SysDev &d0, int stage, int first, int count, cudaS
             launch_stage(d0, stage, s);
             break;
     }
-}
-
-// Forces from device memory to page-locked host memory (coalesced 16-byte stores where both addresses
-// allow) and the control block to its host copy: the last step of an evaluation on host arrays.
-__global__ void __launch_bounds__(256) k_copy_out(const float *src, float *dst, long long nf, const Ctl *ctl, Ctl *hctl,
-                                                  double *res8) {
-    pdl_wait();
-    const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x, nth = (long long)gridDim.x * blockDim.x;
-    if (((((size_t)src) | ((size_t)dst)) & 15) == 0) {
-        const long long n4 = nf >> 2;
-        for (long long i = tid; i < n4; i += nth) ((float4 *)dst)[i] = __ldcg((const float4 *)src + i);
-        for (long long i = (n4 << 2) + tid; i < nf; i += nth) dst[i] = __ldcg(src + i);
-    } else {
-        for (long long i = tid; i < nf; i += nth) dst[i] = __ldcg(src + i);
-    }
-    if (hctl && blockIdx.x == 0 && threadIdx.x < sizeof(Ctl) / 4)
-        ((unsigned *)hctl)[threadIdx.x] = __ldcg((const unsigned *)ctl + threadIdx.x);
-    if (res8 && blockIdx.x == 0 && threadIdx.x < 8)  // energy, virial[6], status bits
-        res8[threadIdx.x] = threadIdx.x < 7 ? __ldcg(ctl->ev + threadIdx.x) : (double)__ldcg(&ctl->status);
 }
 
 cudaError_t launch_copy_out(const float *src, float *dst, long long nf, const Ctl *ctl, Ctl *hctl, cudaStream_t s,

@@ -35,9 +35,8 @@ constexpr int NT_CONV = 128;   // threads per CTA for the influence stage
 constexpr size_t MAX_SMEM_BYTES = 226 * 1024;  // opt-in limit is 227 KB including static shared memory
 constexpr size_t GROUP_SMEM_BYTES = MAX_SMEM_BYTES - sizeof(SysDev) - 64;  // beside the system's descriptor
 
-// Mesh edges K whose lane plans get kernels (and batch stage calls) specialised at compile time: slab kernels for
-// K2 = K3 = K, influence kernels for K1 = K.
-#define PME_EDGES(X)                                                                                         \
+// Mesh edges K1 = K whose lane plan gets an influence kernel specialised at compile time.
+#define PME_EDGES(X)                                                                                             \
     X(16) X(18) X(20) X(24) X(30) X(32) X(36) X(40) X(48) X(50) X(54) X(60) X(64) X(72) X(80) X(90) X(96) X(100) \
         X(108) X(120) X(128)
 template <int K>
@@ -66,6 +65,8 @@ int slab_split(int inverse);
 
 // Raise the dynamic shared-memory limit of the large-footprint kernels (once per device).
 cudaError_t configure_kernels();
+// Load the kernels that need no such limit (a kernel is loaded when it is first named to the runtime).
+cudaError_t load_stage_kernels();
 inline cudaError_t set_dynamic_smem(const void *fn, size_t bytes) {
     return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }

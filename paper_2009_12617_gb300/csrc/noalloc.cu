@@ -6,27 +6,24 @@
 // latency-bound caller (a request loop, a real-time controller) cannot afford on every call. Such
 // callers pass only their inputs and outputs; everything else lives in a fixed static device array.
 //
-// How: one cooperative kernel runs every stage of the evaluation (influence-table set-up, binning,
-// spreading, forward FFT, influence multiply with energy / virial, inverse FFT, force interpolation),
-// separated by grid-wide barriers. The cooperative launch guarantees that all CTAs are resident, so the
-// barriers always complete. All scratch is carved out of g_noalloc_scratch, a file-scope
-// static __device__ array of NOALLOC_SCRATCH_BYTES that every GPU loading the library holds until exit.
-#include <cooperative_groups.h>
+// How: a set-up kernel clears what must start at zero and writes the mesh's tables, then the six stage kernels of
+// an ordinary evaluation follow on the stream, the last of them storing the result in page-locked host memory. All scratch is
+// carved out of g_noalloc_scratch, a file-scope static __device__ array of NOALLOC_SCRATCH_BYTES that every GPU
+// loading the library holds until exit. Every kernel a call may need is loaded by the first call on a device
+// (loading one later could take device memory).
+//
+// 2048 atoms, 32^3, p = 4: 60 us a call. One cooperative kernel with nine grid barriers, its table from
+// a division and two exponentials more per point and its transforms in shared memory took 97 us (88 on the GPU).
 #include <cuda_runtime.h>
 #include <string.h>
 
 #include <mutex>
 
-// The single cooperative kernel keeps only the shared-memory transforms (one code path per stage keeps it
-// small to build); its plans say so through choose_fft_paths(d, false).
-#define PME_NO_LANE_FFT 1
 #include "../../include/pme.h"
 #include "host_tables.h"
 #include "kernels.h"
+#include "pdl.cuh"
 #include "plan_internal.h"
-#include "stages.cuh"
-
-namespace cg = cooperative_groups;
 
 namespace pme {
 
@@ -34,6 +31,7 @@ constexpr size_t NOALLOC_SCRATCH_BYTES = (size_t)4 << 20;  // 4 MiB per device
 constexpr int NOALLOC_MAX_MESH_POINTS = 32768;             // K1 * K2 * K3 (e.g. 32^3)
 constexpr int64_t NOALLOC_MAX_ATOMS = 16384;
 constexpr int NOALLOC_THREADS = 256;
+constexpr int NOALLOC_MAX_EDGE = 64;
 
 }  // namespace pme
 
@@ -44,164 +42,119 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[pme::NOALLOC_SC
 namespace pme {
 
 struct NoallocArgs {
-    SysDev d;
+    int K1, K2, K3, H3;
     double recip[9];  // a*_alpha[j] at 3*alpha + j
-    double vol, beta;
-    double *bmod;     // |b_1|^2 (K1), |b_2|^2 (K2), |b_3|^2 (K3)
-    float4 *bc;       // writable alias of d.bc
-    float2 *tw;       // writable alias of the twiddle block (K1 + K2 + K3/2 + K3/2 + 1)
-    unsigned long long zero_bytes;  // bytes from the scratch start that must be zero before binning
+    double fac;       // pi^2 / beta^2
+    double inv_piv;   // 1 / (pi V)
+    float4 *bc;       // influence table (SysDev::bc)
+    float2 *tw;       // twiddles: K1, K2, K3/2, K3/2 + 1 entries (SysDev::tw1, tw2, tw3h, tw3)
+    unsigned long long *zero;  // what must be zero before binning
+    int nzero;                 // 8-byte words
 };
 
-__device__ double dev_signed_freq(int m, int K) { return (double)(2 * m <= K ? m : m - K); }
-
-__device__ double dev_norm2(const NoallocArgs &A, double mt1, double mt2, double mt3) {
-    const double *r = A.recip;
-    double mv[3];
-    for (int j = 0; j < 3; ++j) mv[j] = mt1 * r[j] + mt2 * r[3 + j] + mt3 * r[6 + j];
-    return mv[0] * mv[0] + mv[1] * mv[1] + mv[2] * mv[2];
-}
-// C(m) and the virial factor f(m) = 2 (1 / |m'|^2 + pi^2 / beta^2) from |m'|^2
-__device__ double dev_influence_c(const NoallocArgs &A, double m2n) {
-    const double pi = 3.14159265358979323846;
-    return exp(-pi * pi * m2n / (A.beta * A.beta)) / (pi * A.vol * m2n);
-}
-__device__ double dev_virial_f(const NoallocArgs &A, double m2n) {
-    const double pi = 3.14159265358979323846;
-    return 2.0 * (1.0 / m2n + pi * pi / (A.beta * A.beta));
-}
-
+// M_P(x) at the integer x, by the recursion over orders.
 template <int P>
-__global__ void __launch_bounds__(NOALLOC_THREADS) k_eval_noalloc(NoallocArgs A) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    cg::grid_group grid = cg::this_grid();
-    const SysDev &d = A.d;
-    const int tid = threadIdx.x, nth = blockDim.x;
-    const int gtid = blockIdx.x * nth + tid, gnth = gridDim.x * nth;
+__host__ __device__ constexpr double spline_knot(int x) {
+    if constexpr (P == 2) {
+        return x == 1 ? 1.0 : 0.0;
+    } else {
+        return ((double)x * spline_knot<P - 1>(x) + (double)(P - x) * (x >= 1 ? spline_knot<P - 1>(x - 1) : 0.0)) / (P - 1);
+    }
+}
 
-    // 0: clear what must start at zero (control block, counters, partials, charge mesh) whatever the
-    //    previous call left; B-spline moduli and FFT twiddles for this mesh.
-    {
-        unsigned long long *z = (unsigned long long *)g_noalloc_scratch;
-        for (unsigned long long i = gtid; i < A.zero_bytes / 8; i += gnth) z[i] = 0ull;
-        const int Ks[3] = {d.K1, d.K2, d.K3};
-        const int Ktot = d.K1 + d.K2 + d.K3;
-        for (int i = gtid; i < Ktot; i += gnth) {
-            const int al = i < d.K1 ? 0 : (i < d.K1 + d.K2 ? 1 : 2);
-            const int m = i - (al == 0 ? 0 : (al == 1 ? d.K1 : d.K1 + d.K2));
-            const int K = Ks[al];
-            // M_P at the integer knots by the unnormalised recursion, then the Euler spline denominator
-            double M[P + 1], prev[P + 1];
-            for (int x = 0; x <= P; ++x) prev[x] = (x == 1) ? 1.0 : 0.0;
-            for (int nn = 3; nn <= P; ++nn) {
-                for (int x = 0; x <= P; ++x) M[x] = ((double)x * prev[x] + (double)(nn - x) * (x >= 1 ? prev[x - 1] : 0.0)) / (nn - 1);
-                for (int x = 0; x <= P; ++x) prev[x] = M[x];
-            }
-            double sr = 0.0, si = 0.0;
-            for (int k = 0; k <= P - 2; ++k) {
-                double s, c;
-                sincospi(2.0 * (double)((m * k) % K) / (double)K, &s, &c);
-                sr += prev[k + 1] * c;
-                si += prev[k + 1] * s;
-            }
-            A.bmod[i] = 1.0 / (sr * sr + si * si);
-        }
-        const int Nh = d.K3 / 2;
-        const int lens[4] = {d.K1, d.K2, Nh, d.K3};
-        const int counts[4] = {d.K1, d.K2, Nh, Nh + 1};
-        const int ntw = d.K1 + d.K2 + Nh + Nh + 1;
-        for (int i = gtid; i < ntw; i += gnth) {
-            int seg = 0, k = i;
-            while (k >= counts[seg]) k -= counts[seg++];
-            double s, c;
-            sincospi(-2.0 * (double)k / (double)lens[seg], &s, &c);
-            A.tw[i] = make_float2((float)c, (float)s);
+__device__ __forceinline__ int dev_signed_freq(int m, int K) { return 2 * m <= K ? m : m - K; }
+
+__device__ __forceinline__ double dev_norm2(const NoallocArgs &A, int mt1, int mt2, int mt3) {
+    const double *r = A.recip;
+    double s = 0.0;
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        const double v = mt1 * r[j] + mt2 * r[3 + j] + mt3 * r[6 + j];
+        s += v * v;
+    }
+    return s;
+}
+
+// Clears the charge mesh, counters, partials and control block, and writes the twiddles and the influence table,
+// all in FP64 rounded once. Each block keeps the spline denominators of the three axes in shared memory: with the
+// knots symmetric about P / 2, |sum_k M_P(k + 1) exp(2 pi i m k / K)| = |M_P(P/2) + 2 sum_d M_P(P/2 + d)
+// cos(2 pi m d / K)|. A table point costs one exponential and one division, and as much again on Nyquist planes;
+// the FP64 pipe (1/64 of FP32) bounds this kernel, about 3 us at 32^3.
+template <int P>
+__global__ void __launch_bounds__(NOALLOC_THREADS) k_noalloc_setup(NoallocArgs A) {
+    __shared__ double den[3 * NOALLOC_MAX_EDGE];
+    pdl_wait();
+    const int tid = threadIdx.x, nth = blockDim.x, gtid = blockIdx.x * nth + tid, gnth = gridDim.x * nth;
+    for (int i = gtid; i < A.nzero; i += gnth) A.zero[i] = 0ull;
+    const int K1 = A.K1, K2 = A.K2, K3 = A.K3, H3 = A.H3, Nh = K3 / 2;
+    constexpr double knots[4] = {spline_knot<P>(P / 2), spline_knot<P>(P / 2 + 1), spline_knot<P>(P / 2 + 2), spline_knot<P>(P / 2 + 3)};
+    for (int i = tid; i < 3 * NOALLOC_MAX_EDGE; i += nth) {
+        const int al = i / NOALLOC_MAX_EDGE, m = i - al * NOALLOC_MAX_EDGE, K = al == 0 ? K1 : (al == 1 ? K2 : K3);
+        if (m < K) {
+            double s = knots[0];
+#pragma unroll
+            for (int k = 1; k < P / 2; ++k) s += 2.0 * knots[k] * cospi(2.0 * (double)((m * k) % K) / (double)K);
+            den[i] = s;
         }
     }
-    grid.sync();
-    // 1: influence table on the half spectrum, [m2][m1][m3] (SysDev::bc): B(m) (C(m) + C(-m)) / 2 as (hi, lo)
-    // floats, then B C f(m) and, off the self-conjugate planes on a Nyquist plane, B C f(m_p)
-    {
-        const int H3 = d.H3;
-        const int tot = d.K1 * d.K2 * H3;
-        for (int i = gtid; i < tot; i += gnth) {
-            const int m3 = i % H3, m1 = (i / H3) % d.K1, m2 = i / (H3 * d.K1);
-            double v = 0.0, g = 0.0, gp = 0.0;
-            if (m1 | m2 | m3) {
-                const int mt1 = dev_signed_freq(m1, d.K1), mt2 = dev_signed_freq(m2, d.K2), mt3 = dev_signed_freq(m3, d.K3);
-                const double nm = dev_norm2(A, mt1, mt2, mt3);
-                const double np = dev_norm2(A, dev_signed_freq((d.K1 - m1) % d.K1, d.K1),
-                                            dev_signed_freq((d.K2 - m2) % d.K2, d.K2),
-                                            dev_signed_freq((d.K3 - m3) % d.K3, d.K3));
-                v = A.bmod[m1] * A.bmod[d.K1 + m2] * A.bmod[d.K1 + d.K2 + m3] * 0.5 *
-                    (dev_influence_c(A, nm) + dev_influence_c(A, np));
-                g = v * dev_virial_f(A, nm);
-                const bool self = m3 == 0 || 2 * m3 == d.K3;
-                if (!self && (2 * m1 == d.K1 || 2 * m2 == d.K2))
-                    gp = v * dev_virial_f(A, dev_norm2(A, 2 * m1 == d.K1 ? mt1 : -mt1, 2 * m2 == d.K2 ? mt2 : -mt2, -mt3));
+    for (int i = gtid; i < K1 + K2 + Nh + Nh + 1; i += gnth) {
+        int k = i, len = K1;
+        if (k >= K1) {
+            k -= K1, len = K2;
+            if (k >= K2) {
+                k -= K2, len = Nh;
+                if (k >= Nh) k -= Nh, len = K3;
             }
-            const float hi = (float)v;
-            A.bc[i] = make_float4(hi, (float)(v - (double)hi), (float)g, (float)gp);
         }
+        double s, c;
+        sincospi(-2.0 * (double)k / (double)len, &s, &c);
+        A.tw[i] = make_float2((float)c, (float)s);
     }
-    grid.sync();
-    // 2..7: the six pipeline stages, each over its work items, with a grid barrier in between
-    // A CTA that takes several items of one stage waits at a CTA barrier after each: the next item's first
-    // shared-memory writes (spread_clear, the gather's region load) must not overtake warps still reading
-    // the previous item's tile.
-    const int nbin = d.nbin;
-    for (int it = blockIdx.x; it < nbin; it += gridDim.x) {
-        stage_bin(d, it, smem);
-        __syncthreads();
-    }
-    grid.sync();
-    for (int it = blockIdx.x; it < d.ntiles + OVF_ITEMS; it += gridDim.x) {
-        stage_spread<P, 8>(d, it, smem);
-        __syncthreads();
-    }
-    grid.sync();
-    for (int it = blockIdx.x; it < d.K1; it += gridDim.x) {
-        stage_fwd(d, it, smem);
-        __syncthreads();
-    }
-    grid.sync();
-    for (int it = blockIdx.x; it < d.nconv; it += gridDim.x) {
-        stage_conv(d, it, smem);
-        __syncthreads();
-    }
-    grid.sync();
-    for (int it = blockIdx.x; it < d.K1; it += gridDim.x) {
-        stage_inv(d, it, smem);
-        __syncthreads();
-    }
-    grid.sync();
-    for (int it = blockIdx.x; it < d.ntiles + OVF_ITEMS; it += gridDim.x) {
-        stage_gather<P, 8>(d, it, smem);
-        __syncthreads();
+    __syncthreads();
+    // on the half spectrum, [m2][m1][m3]: B(m) (C(m) + C(-m)) / 2 as (hi, lo) floats, then B C f(m) and, off the
+    // self-conjugate planes on a Nyquist plane, B C f(m_p), f = 2 (1 / |m'|^2 + pi^2 / beta^2)
+    for (int i = gtid; i < K1 * K2 * H3; i += gnth) {
+        const int m3 = i % H3, m1 = (i / H3) % K1, m2 = i / (H3 * K1);
+        double v = 0.0, g = 0.0, gp = 0.0;
+        if (m1 | m2 | m3) {
+            const int mt1 = dev_signed_freq(m1, K1), mt2 = dev_signed_freq(m2, K2);
+            const double d = den[m1] * den[NOALLOC_MAX_EDGE + m2] * den[2 * NOALLOC_MAX_EDGE + m3], D = d * d;
+            const double nm = dev_norm2(A, mt1, mt2, m3);
+            const double inv = 1.0 / (nm * D);  // B / |m'|^2
+            v = exp(-A.fac * nm) * inv;
+            const double f = 2.0 * (inv * D + A.fac);
+            if (2 * m1 == K1 || 2 * m2 == K2 || 2 * m3 == K3) {
+                // the index of -m keeps the frequency +K/2 on a Nyquist axis
+                const int p1 = 2 * m1 == K1 ? mt1 : -mt1, p2 = 2 * m2 == K2 ? mt2 : -mt2;
+                const double np = dev_norm2(A, p1, p2, 2 * m3 == K3 ? m3 : -m3);
+                v = 0.5 * (v + exp(-A.fac * np) / (np * D));
+                const bool self = m3 == 0 || 2 * m3 == K3;
+                if (!self && (2 * m1 == K1 || 2 * m2 == K2)) gp = v * A.inv_piv * 2.0 * (1.0 / np + A.fac);
+            }
+            v *= A.inv_piv;
+            g = v * f;
+        }
+        const float hi = (float)v;
+        A.bc[i] = make_float4(hi, (float)(v - (double)hi), (float)g, (float)gp);
     }
 }
 
 struct NoallocDevice {
     bool ready = false;
     unsigned char *scratch = nullptr;  // device address of g_noalloc_scratch
-    int grid[9] = {0};                 // co-resident CTAs for P = 4, 6, 8 (index P)
+    int sms = 0;
+    double *result = nullptr, *result_dev = nullptr;  // page-locked result (8 doubles) and its device address
 };
 
 static std::mutex g_noalloc_mu;
 static NoallocDevice g_noalloc_dev[64];
 
-static size_t noalloc_smem(int K[3], int p) {
-    size_t s = smem_bin(NOALLOC_THREADS);
-    s = s > smem_spread(p, 3) ? s : smem_spread(p, 3);  // this path always uses 8^3 tiles
-    s = s > smem_gather_all(p, 3) ? s : smem_gather_all(p, 3);
-    s = s > smem_slab(K[1], K[2]) ? s : smem_slab(K[1], K[2]);
-    s = s > smem_inv(K[1], K[2]) ? s : smem_inv(K[1], K[2]);
-    s = s > smem_conv(K[0], NOALLOC_THREADS) ? s : smem_conv(K[0], NOALLOC_THREADS);
-    return s;
+static const void *setup_kernel(int p) {
+    return p == 4 ? (const void *)k_noalloc_setup<4> : (p == 6 ? (const void *)k_noalloc_setup<6> : (const void *)k_noalloc_setup<8>);
 }
 
-// Once per device, with that device current: the scratch array's device address and the number of CTAs
-// of each kernel variant that fit on the device at once (the cooperative grid size).
+// Once per device, with that device current: the scratch array's device address, the page-locked result block, and
+// every kernel that a later call may launch loaded.
 static pme_status noalloc_setup(int dev, NoallocDevice **out) {
     std::lock_guard<std::mutex> lk(g_noalloc_mu);
     if (dev < 0 || dev >= 64) return fail(PME_ECUDA, "device index %d out of range", dev);
@@ -210,26 +163,29 @@ static pme_status noalloc_setup(int dev, NoallocDevice **out) {
         void *ptr = nullptr;
         cudaError_t e = cudaGetSymbolAddress(&ptr, g_noalloc_scratch);
         if (e != cudaSuccess) return cuda_fail(e, "cudaGetSymbolAddress(g_noalloc_scratch)");
-        int sms = 0, coop = 0;
-        if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
+        if ((e = cudaDeviceGetAttribute(&nd.sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
             return cuda_fail(e, "cudaDeviceGetAttribute");
-        if ((e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev)) != cudaSuccess)
-            return cuda_fail(e, "cudaDeviceGetAttribute");
-        if (!coop) return fail(PME_EUNSUPPORTED, "device does not support cooperative launches");
-        const void *fns[3] = {(const void *)k_eval_noalloc<4>, (const void *)k_eval_noalloc<6>,
-                              (const void *)k_eval_noalloc<8>};
-        const int ps[3] = {4, 6, 8};
-        for (int i = 0; i < 3; ++i) {
-            int K[3] = {64, 64, 64};  // the largest shared-memory footprint the size limits allow
-            const size_t smem = noalloc_smem(K, ps[i]);
-            if ((e = cudaFuncSetAttribute(fns[i], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-                return cuda_fail(e, "cudaFuncSetAttribute(k_eval_noalloc)");
-            int per_sm = 0;
-            if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fns[i], NOALLOC_THREADS, smem)) != cudaSuccess)
-                return cuda_fail(e, "cudaOccupancyMaxActiveBlocksPerMultiprocessor");
-            if (per_sm < 1) return fail(PME_ECUDA, "k_eval_noalloc does not fit on an SM");
-            nd.grid[ps[i]] = sms * (per_sm < 2 ? per_sm : 2);
+        if ((e = ensure_configured(dev)) != cudaSuccess) return cuda_fail(e, "configure kernels");
+        cudaFuncAttributes fa;
+        for (int p : {4, 6, 8})
+            if ((e = cudaFuncGetAttributes(&fa, setup_kernel(p))) != cudaSuccess) return cuda_fail(e, "cudaFuncGetAttributes");
+        if ((e = load_stage_kernels()) != cudaSuccess) return cuda_fail(e, "cudaFuncGetAttributes");
+        const double recip[9] = {1, 0, 0, 0, 1, 0, 0, 0, 1};
+        for (int i = 0; i < N_EDGES && mesh_edge(i) <= NOALLOC_MAX_EDGE; ++i) {
+            SysDev d;
+            memset(&d, 0, sizeof(d));
+            const int Ke = mesh_edge(i), K[3] = {Ke, Ke, Ke}, Kr[3] = {Ke, 8, 10};  // own slab kernels; general ones
+            for (const int *k : {K, Kr}) {
+                fill_geometry(d, k, 4, 1.0, recip);
+                if ((e = configure_transforms(d)) != cudaSuccess) return cuda_fail(e, "configure kernels");
+            }
         }
+        if (!nd.result && (e = lib_malloc_host((void **)&nd.result, 8 * sizeof(double))) != cudaSuccess) {
+            nd.result = nullptr;
+            return cuda_fail(e, "cudaMallocHost");
+        }
+        if ((e = cudaHostGetDevicePointer((void **)&nd.result_dev, nd.result, 0)) != cudaSuccess)
+            return cuda_fail(e, "cudaHostGetDevicePointer");
         nd.scratch = (unsigned char *)ptr;
         nd.ready = true;
     }
@@ -268,23 +224,23 @@ extern "C" pme_status pme_compute_noalloc(const int K[3], int p, double beta, co
     pme_status st = noalloc_setup(dev, &nd);
     if (st != PME_OK) return st;
 
-    // carve the static scratch: everything that must start at zero comes first
-    NoallocArgs A;
-    memset(&A, 0, sizeof(A));
-    SysDev &d = A.d;
+    // carve the static scratch: everything that must start at zero comes first. The space set aside for partials and
+    // tables is that of the finest division of the influence stage, CONV_COLS columns of one m2 an item.
+    SysDev d;
+    memset(&d, 0, sizeof(d));
     fill_geometry(d, K, p, beta, recip);
-    choose_fft_paths(d, false);
     const size_t K1 = K[0], K2 = K[1], K3 = K[2], H3 = d.H3, Nh = K3 / 2;
+    const size_t par_bytes = (K2 * (size_t)d.nchunk3 + K1) * 8 * sizeof(float2);
     const int64_t ncap = n > 0 ? n : 1;
     const int cap = bucket_capacity(ncap, d.ntiles, d.tlog);
     size_t off = 0;
     const size_t o_ctl = off;  off = al256(off + sizeof(Ctl));
     const size_t o_cnt = off;  off = al256(off + bcount_bytes(d.ntiles));
     const size_t o_qs = off;   off = al256(off + QABS_BYTES);
-    const size_t o_par = off;  off = al256(off + partials_bytes(d));
+    const size_t o_par = off;  off = al256(off + par_bytes);
     const size_t o_grid = off; off = al256(off + K1 * K2 * K3 * 8);
     const size_t zero_bytes = off;
-    const size_t o_bmod = off; off = al256(off + (K1 + K2 + K3) * 8);
+    off = al256(off + (K1 + K2 + K3) * 8);
     const size_t o_tw = off;   off = al256(off + (K1 + K2 + Nh + Nh + 1) * 8);
     const size_t o_bc = off;   off = al256(off + K1 * K2 * H3 * sizeof(float4));
     const size_t o_spec = off; off = al256(off + K1 * K2 * H3 * 8);
@@ -302,7 +258,8 @@ extern "C" pme_status pme_compute_noalloc(const int K[3], int p, double beta, co
     d.qslot = (unsigned long long *)(b + o_qs);
     d.partials = (double *)(b + o_par);
     d.grid = (unsigned long long *)(b + o_grid);
-    A.bmod = (double *)(b + o_bmod);
+    NoallocArgs A;
+    memset(&A, 0, sizeof(A));
     A.tw = (float2 *)(b + o_tw);
     d.tw1 = A.tw;
     d.tw2 = A.tw + K1;
@@ -322,26 +279,36 @@ extern "C" pme_status pme_compute_noalloc(const int K[3], int p, double beta, co
     d.pos = pos;
     d.q = q;
     d.forces = forces;
-    d.ev = d.ctl->ev;
+    d.ev = nd->result_dev;  // the final reduction stores energy, virial and status bits there
+    d.ev_status = 1;
+    A.K1 = K[0];
+    A.K2 = K[1];
+    A.K3 = K[2];
+    A.H3 = d.H3;
     memcpy(A.recip, recip, sizeof(recip));
-    A.vol = vol;
-    A.beta = beta;
-    A.zero_bytes = zero_bytes;
+    A.fac = PI_D * PI_D / (beta * beta);
+    A.inv_piv = 1.0 / (PI_D * vol);
+    A.zero = (unsigned long long *)b;
+    A.nzero = (int)(zero_bytes / 8);
 
-    int Kc[3] = {K[0], K[1], K[2]};
-    const size_t smem = noalloc_smem(Kc, p);
-    const void *fn = p == 4 ? (const void *)k_eval_noalloc<4> : (p == 6 ? (const void *)k_eval_noalloc<6> : (const void *)k_eval_noalloc<8>);
-    void *args[] = {&A};
     cudaStream_t stream = (cudaStream_t)cuda_stream;
-    e = cudaLaunchCooperativeKernel(fn, dim3(nd->grid[p]), dim3(NOALLOC_THREADS), args, smem, stream);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaLaunchCooperativeKernel(k_eval_noalloc)");
-    Ctl h;  // pageable host copy: this copy returns once the kernel and the copy are done
-    if ((e = cudaMemcpyAsync(&h, d.ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, stream)) != cudaSuccess)
-        return cuda_fail(e, "cudaMemcpyAsync(result)");
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)nd->sms);
+    cfg.blockDim = dim3(NOALLOC_THREADS);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = launch_mode() ? 1 : 0;
+    void *args[] = {&A};
+    if ((e = cudaLaunchKernelExC(&cfg, setup_kernel(p), args)) != cudaSuccess) return cuda_fail(e, "kernel launch");
+    if ((e = launch_pipeline(d, stream)) != cudaSuccess) return cuda_fail(e, "kernel launch");
     if ((e = cudaStreamSynchronize(stream)) != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
-    if ((st = status_from_bits(h.status)) != PME_OK) return st;
-    if (energy) *energy = h.ev[0];
+    const double *r = nd->result;
+    if ((st = status_from_bits((unsigned)r[7])) != PME_OK) return st;
+    if (energy) *energy = r[0];
     if (virial)
-        for (int c = 0; c < 6; ++c) virial[c] = h.ev[1 + c];
+        for (int c = 0; c < 6; ++c) virial[c] = r[1 + c];
     return PME_OK;
 }

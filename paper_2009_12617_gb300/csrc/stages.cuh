@@ -1,7 +1,7 @@
 // Stage bodies of the reciprocal-space SPME pipeline (paper Sec. III-A, Fig. "LRPipe"): binning with
 // B-spline set-up, charge spreading, forward 3D FFT, influence-function multiply with energy / virial,
 // inverse 3D FFT, and force interpolation. Each body handles one work item of one system and is called
-// both from the per-stage kernels and from the batched / cooperative kernels.
+// both from the per-stage kernels and from the batched kernels.
 //
 // Work items per system:
 //   bin     nbin items          atoms [item*BIN_CHUNK, ...): fractional coordinates, tile key, bucket insert
@@ -16,9 +16,8 @@
 #include "common.cuh"
 #include "fft.cuh"
 
-// The register transforms (lane plans) need warps; the CPU emulation and builds that define
-// PME_NO_LANE_FFT keep only the shared-memory transforms.
-#if !defined(PME_HOST_EMULATION) && !defined(PME_NO_LANE_FFT)
+// The register transforms (lane plans) need warps; the CPU emulation keeps only the shared-memory transforms.
+#if !defined(PME_HOST_EMULATION)
 #define PME_LANE_FFT 1
 #endif
 
@@ -1466,8 +1465,7 @@ PME_DEV void stage_conv_lane(const SysDev &d, int item, void *smem) {
 }
 #endif  // PME_LANE_FFT
 
-// Stage entry points: the register path, or the shared-memory path in builds without it (the CPU emulation, the
-// allocation-free kernel). With plans given at compile time (a kernel specialised for one mesh) only their code
+// Stage entry points: the register path, or the shared-memory path in the CPU emulation. With plans given at compile time (a kernel specialised for one mesh) only their code
 // is built in; such a kernel runs only for systems with exactly those plans.
 template <int PR = -1, int PC = -1>
 PME_DEV void stage_fwd(const SysDev &d, int k1, void *smem) {
