@@ -17,7 +17,7 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 INCLUDE = os.path.join(ROOT, "include")
 LIB_NAME = "libpme_gb300.so"
-SOURCES = ["fwd.cu", "inv.cu", "conv.cu", "kernels.cu", "group.cu", "batch.cu", "plan.cu", "server.cu", "noalloc.cu", "probe.cu", "realspace.cu", "tune.cu", "md.cu", "tc_dft.cu", "slab.cu"]
+SOURCES = ["batch.cu", "fwd.cu", "fwd2.cu", "inv.cu", "inv2.cu", "conv.cu", "kernels.cu", "group.cu", "plan.cu", "server.cu", "noalloc.cu", "probe.cu", "realspace.cu", "tune.cu", "md.cu", "tc_dft.cu", "slab.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

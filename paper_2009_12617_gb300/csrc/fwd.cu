@@ -1,53 +1,38 @@
-// The forward slab stage kernels, for one system and for a group of systems (batches, server waves): one kernel per
-// mesh edge K2 = K3 with that edge's lane plans at compile time (each holds only its plans' code, which keeps it
-// small enough for the instruction caches), and one that picks the plans at run time for other meshes.
-#include <cuda_runtime.h>
-
-#include "group.h"
-#include "kernels.h"
-#include "pdl.cuh"
-#include "stages.cuh"
+// The forward slab stage kernels (slab_kernels.cuh): those for every second K2 (fwd2.cu has the others), the ones
+// that pick their plans at run time, and the choice among them.
+#include "slab_kernels.cuh"
 
 namespace pme {
 
-template <int PR, int PC>
-__global__ void __launch_bounds__(NT_SLAB) k_fwd(SysDev d) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    PdlScope pdl(d.pdl_late);
-    stage_fwd<PR, PC>(d, d.item0 + blockIdx.x, smem);
-}
+struct FwdStage {
+    template <int PR, int PC>
+    static __device__ __forceinline__ void run(const SysDev &d, int k1, void *smem) {
+        stage_fwd<PR, PC>(d, k1, smem);
+    }
+};
 
-template <int PR, int PC>
-__global__ void __launch_bounds__(NT_SLAB) k_fwd_g(GroupArgs a) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ SysDev sd;
-    PdlScope pdl(a.late);
-    const int item = group_load(a, sd);
-    stage_fwd<PR, PC>(sd, item, smem);
+static const SlabTable<FwdStage, 0> &table() {
+    static const SlabTable<FwdStage, 0> t;
+    return t;
 }
+StageKernel fwd_kernel_odd(int i2, int i3);
+GroupKernel fwd_group_kernel_odd(int i2, int i3);
+cudaError_t configure_fwd_group_kernels_odd();
 
-#define PME_PICK(K, kernel) \
-    if (d.lp_rows == Edge<K>::PR && d.lp_cols == Edge<K>::PC) return kernel<Edge<K>::PR, Edge<K>::PC>;
 StageKernel fwd_kernel(const SysDev &d) {
-#define PME_PICK_K(K) PME_PICK(K, k_fwd)
-    PME_EDGES(PME_PICK_K)
-#undef PME_PICK_K
-    return k_fwd<-1, -1>;
+    const int i2 = edge_index(d.K2), i3 = edge_index(d.K3);
+    const StageKernel k = i2 & 1 ? fwd_kernel_odd(i2, i3) : table().find(i2, i3);
+    return k ? k : k_slab<FwdStage, -1, -1>;
 }
 GroupKernel fwd_group_kernel(const SysDev &d) {
-#define PME_PICK_K(K) PME_PICK(K, k_fwd_g)
-    PME_EDGES(PME_PICK_K)
-#undef PME_PICK_K
-    return k_fwd_g<-1, -1>;
+    const int i2 = edge_index(d.K2), i3 = edge_index(d.K3);
+    const GroupKernel k = i2 & 1 ? fwd_group_kernel_odd(i2, i3) : table().find_group(i2, i3);
+    return k ? k : k_slab_g<FwdStage, -1, -1>;
 }
-
 cudaError_t configure_fwd_group_kernels() {
-    cudaError_t e;
-#define PME_CFG_K(K) \
-    if ((e = set_dynamic_smem((const void *)k_fwd_g<Edge<K>::PR, Edge<K>::PC>, GROUP_SMEM_BYTES)) != cudaSuccess) return e;
-    PME_EDGES(PME_CFG_K)
-#undef PME_CFG_K
-    return set_dynamic_smem((const void *)k_fwd_g<-1, -1>, GROUP_SMEM_BYTES);
+    for (cudaError_t e : {configure_fwd_group_kernels_odd(), table().configure_group()})
+        if (e != cudaSuccess) return e;
+    return set_dynamic_smem((const void *)k_slab_g<FwdStage, -1, -1>, GROUP_SMEM_BYTES);
 }
 
 }  // namespace pme
