@@ -353,6 +353,52 @@ PME_DEV DF df_add(DF a, DF b) {
 }
 
 // ---------------------------------------------------------------------------------------------------------
+// Pairs of FP32 numbers: on the GPU one 64-bit register, and one instruction works on both (each half rounded as
+// the scalar instruction would).
+#if defined(PME_HOST_EMULATION)
+struct F2 {
+    float x, y;
+};
+inline F2 f2(float x, float y) { return F2{x, y}; }
+inline float2 f2_get(F2 a) { return make_float2(a.x, a.y); }
+inline F2 f2_fma(F2 a, F2 b, F2 c) { return F2{fmaf(a.x, b.x, c.x), fmaf(a.y, b.y, c.y)}; }
+inline F2 f2_mul(F2 a, F2 b) { return F2{a.x * b.x, a.y * b.y}; }
+inline F2 f2_add(F2 a, F2 b) { return F2{a.x + b.x, a.y + b.y}; }
+#else
+struct F2 {
+    unsigned long long v;
+};
+__device__ __forceinline__ F2 f2(float x, float y) {
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(x), "f"(y));
+    return r;
+}
+__device__ __forceinline__ float2 f2_get(F2 a) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a.v));
+    return r;
+}
+__device__ __forceinline__ F2 f2_fma(F2 a, F2 b, F2 c) {
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+__device__ __forceinline__ F2 f2_mul(F2 a, F2 b) {
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 f2_add(F2 a, F2 b) {
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+#endif
+PME_DEV F2 f2_all(float x) { return f2(x, x); }
+// a - b: the product with -1 is exact
+PME_DEV F2 f2_sub(F2 a, F2 b) { return f2_fma(b, f2_all(-1.0f), a); }
+
+// ---------------------------------------------------------------------------------------------------------
 // Scaled fractional coordinate of one position along dimension al (paper Sec. III-A "Charge Spreading":
 // an atom sits at a fractional position between mesh points). u = sum_j r_j C[j][al] is formed from exact
 // FP32 products (TwoProd via fma) and TwoSum, so w = u - floor(u) carries no FP32 rounding of u itself

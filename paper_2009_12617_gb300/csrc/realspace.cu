@@ -261,39 +261,6 @@ __device__ __forceinline__ float mufu_rsqrt(float x) {
     return y;
 }
 
-// Pairs of FP32 numbers in one 64-bit register: one instruction works on both.
-struct F2 {
-    unsigned long long v;
-};
-__device__ __forceinline__ F2 f2(float x, float y) {
-    F2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(x), "f"(y));
-    return r;
-}
-__device__ __forceinline__ float2 f2_get(F2 a) {
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a.v));
-    return r;
-}
-__device__ __forceinline__ F2 f2_fma(F2 a, F2 b, F2 c) {
-    F2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
-    return r;
-}
-__device__ __forceinline__ F2 f2_mul(F2 a, F2 b) {
-    F2 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
-    return r;
-}
-__device__ __forceinline__ F2 f2_add(F2 a, F2 b) {
-    F2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
-    return r;
-}
-__device__ __forceinline__ F2 f2_all(float x) { return f2(x, x); }
-// a - b: the product with -1 is exact
-__device__ __forceinline__ F2 f2_sub(F2 a, F2 b) { return f2_fma(b, f2_all(-1.0f), a); }
-
 // exp(x^2) erfc(x) for x >= 0 as t Q(t), t = 1 / (1 + 2 x / 5), Q the degree-10 polynomial that interpolates
 // exp(x^2) erfc(x) / t at the Chebyshev nodes of t in (0, 1] (fitted in 40-digit arithmetic; largest relative
 // error 1.2e-8, below FP32 rounding). x04 = 2 x / 5.

@@ -162,6 +162,17 @@ PME_DEV void fix_split(float v, int &h, int &l) {
     const float r = fmaf(-(t - M), 1048576.0f, v);
     l = float_bits(r + M) - 0x4B400000;
 }
+// The same for two values at once.
+PME_DEV void fix_split2(F2 v, int &h0, int &l0, int &h1, int &l1) {
+    const float M = 12582912.0f;
+    const F2 t = f2_fma(v, f2_all(9.5367431640625e-07f), f2_all(M));
+    const F2 l = f2_add(f2_fma(f2_add(t, f2_all(-M)), f2_all(-1048576.0f), v), f2_all(M));
+    const float2 th = f2_get(t), tl = f2_get(l);
+    h0 = float_bits(th.x) - 0x4B400000;
+    h1 = float_bits(th.y) - 0x4B400000;
+    l0 = float_bits(tl.x) - 0x4B400000;
+    l1 = float_bits(tl.y) - 0x4B400000;
+}
 PME_DEV unsigned long long fix_join(long long h, long long l) { return (unsigned long long)(h * 1048576ll + l); }
 
 // ---------------------------------------------------------------------------------------------------------
@@ -365,6 +376,16 @@ PME_DEV void spread_clear(void *smem) {
     for (int i = PME_TID; i < SpreadSmem<P, T>::VOLP / 2; i += PME_NTH) z[i] = make_int4(0, 0, 0, 0);
 }
 
+// p[i] += v in shared memory: on the GPU a reduction on a 32-bit shared-window address.
+#if defined(PME_HOST_EMULATION)
+inline void shared_add(int *p, int i, int v) { p[i] += v; }
+#else
+__device__ __forceinline__ unsigned smem_u32(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void shared_add(int *p, int i, int v) {
+    asm volatile("red.shared.add.s32 [%0], %1;" ::"r"(smem_u32(p) + 4u * (unsigned)i), "r"(v) : "memory");
+}
+#endif
+
 // One lane's share of an atom on the warp-lane path: points (jA, j2, j3) and (jA + 2, j2, j3) below the
 // atom's highest support point, jA = lane / 16, j2 = lane / 4 mod 4, j3 = lane mod 4. The value added is
 // rn(rn(rn(q th1) 2^40 th2) th3), equal to the two-thread and global paths' rn(rn(rn(q th1) th2) 2^40 th3)
@@ -395,19 +416,17 @@ struct Lanes4 {
     }
     void add(const Lane4 &w) const {
         constexpr int PL = SpreadLayout<P, T>::PL;
-        int h, l;
-        fix_split((w.u.x * w.t2) * w.t3, h, l);
-        s.hi[w.i] += h;
-        s.lo[w.i] += l;
-        fix_split((w.u.y * w.t2) * w.t3, h, l);
-        s.hi[w.i - 2 * PL] += h;
-        s.lo[w.i - 2 * PL] += l;
+        int h0, l0, h1, l1;
+        fix_split2(f2_mul(f2_mul(f2(w.u.x, w.u.y), f2_all(w.t2)), f2_all(w.t3)), h0, l0, h1, l1);
+        s.hi[w.i] += h0;
+        s.lo[w.i] += l0;
+        s.hi[w.i - 2 * PL] += h1;
+        s.lo[w.i - 2 * PL] += l1;
     }
 };
 #else
 // GPU: 32-bit shared-window addresses computed once per lane, so each load or reduction costs one add
 // instead of 64-bit generic pointer arithmetic
-PME_DEV unsigned smem_u32(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
 template <int P, int T>
 struct Lanes4 {
     static constexpr unsigned DLO = 4u * SpreadLayout<P, T>::VOLP;  // lo - hi, bytes
@@ -436,13 +455,12 @@ struct Lanes4 {
     }
     PME_DEV void add(const Lane4 &w) const {
         const unsigned ad = (unsigned)w.i;
-        int h, l;
-        fix_split((w.u.x * w.t2) * w.t3, h, l);
-        red(ad, h);
-        red(ad + DLO, l);
-        fix_split((w.u.y * w.t2) * w.t3, h, l);
-        red(ad - D2, h);
-        red(ad + DLO - D2, l);
+        int h0, l0, h1, l1;
+        fix_split2(f2_mul(f2_mul(f2(w.u.x, w.u.y), f2_all(w.t2)), f2_all(w.t3)), h0, l0, h1, l1);
+        red(ad, h0);
+        red(ad + DLO, l0);
+        red(ad - D2, h1);
+        red(ad + DLO - D2, l1);
     }
 };
 #endif
@@ -582,11 +600,19 @@ PME_DEV void stage_spread(const SysDev &d, int item, void *smem, bool cleared = 
                     const float c = ra.w * t1 * th2[j2] * FIX_SCALE;
                     const int row = (l1 - j1) * PL + (l2 - j2) * R + l3;
 #pragma unroll
-                    for (int j3 = 0; j3 < P; ++j3) {
+                    for (int j3 = 0; j3 + 1 < P; j3 += 2) {  // two points per paired instruction
+                        int h0, l0, h1, l1;
+                        fix_split2(f2_mul(f2_all(c), f2(th3[j3], th3[j3 + 1])), h0, l0, h1, l1);
+                        shared_add(hi, row - j3, h0);
+                        shared_add(lo, row - j3, l0);
+                        shared_add(hi, row - j3 - 1, h1);
+                        shared_add(lo, row - j3 - 1, l1);
+                    }
+                    if (P & 1) {
                         int h, l;
-                        fix_split(c * th3[j3], h, l);
-                        atomic_add_i32(hi + row - j3, h);
-                        atomic_add_i32(lo + row - j3, l);
+                        fix_split(c * th3[P - 1], h, l);
+                        shared_add(hi, row - P + 1, h);
+                        shared_add(lo, row - P + 1, l);
                     }
                 }
             }
