@@ -112,15 +112,18 @@ inline int choose_k1_pieces(const SysDev &d, int sms) {
     return best;
 }
 
-// Tile edge for n atoms on a GPU with `sms` SMs. 16^3 tiles halve the halo each tile adds to the global
-// mesh (a region of (16 + p - 1)^3 points per 4096 instead of (8 + p - 1)^3 per 512) and hold enough atoms
-// per residue class for the dealt order to avoid shared-memory bank conflicts, but there are 8 times fewer
-// of them. They pay when there are still at least two per SM and they hold about 256 atoms or more (128^3,
-// 262144 atoms, p = 6: 144 vs 151 us per evaluation on GB300); otherwise 8^3 tiles (many light CTAs) are
-// faster. Results do not depend on the edge.
-inline int choose_tile_log(int64_t n, const int K[3], int sms) {
+// Tile edge for n atoms at order p on a GPU with `sms` SMs. 16^3 tiles halve the halo each tile adds to the global
+// mesh (a region of (16 + p - 1)^3 points per 4096 instead of (8 + p - 1)^3 per 512) and there are 8 times fewer of
+// them, so they pay as soon as there is about one per SM, at any density measured (from 48 atoms a tile; below 32,
+// 8^3 is kept). us per evaluation with 8^3 / 16^3 tiles, 152 SMs: p = 6 at 80 x 80 x 96 (150 tiles, 60000 atoms)
+// 63 / 56, 90 x 96 x 100 (252 tiles) with 12000, 50001 and 80001 atoms 62 / 57, 69 / 58, 73 / 65, 128^3 with 25000 and
+// 262144 atoms 109 / 84, 147 / 126; p = 8 at 80 x 80 x 96 90 / 73; but 80^3 (125 tiles, 120000 atoms) 67 / 79. At p = 4
+// the halo is thin and the 8^3 spreading kernel free of bank conflicts, so that it takes a few more tiles: 72 x 80 x 96
+// (150 tiles, 90000 atoms) 48 / 52, 72 x 80 x 100 (175 tiles) 45.9 / 44.9, 128^3 98 / 90. Results do not depend on the edge.
+inline int choose_tile_log(int64_t n, const int K[3], int sms, int p = 4) {
     const int64_t t16 = (int64_t)((K[0] + 15) / 16) * ((K[1] + 15) / 16) * ((K[2] + 15) / 16);
-    if (sms > 0 && t16 >= 2 * (int64_t)sms && n >= 256 * t16) return TILE_MAX_LOG;
+    const int64_t want = p == 4 ? sms + sms / 8 : sms - sms / 16;
+    if (sms > 0 && t16 >= want && n >= 32 * t16) return TILE_MAX_LOG;
     return TILE_MIN_LOG;
 }
 

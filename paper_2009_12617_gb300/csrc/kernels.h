@@ -10,6 +10,7 @@
 
 namespace pme {
 
+constexpr int GB300_SMS = 152;
 constexpr int NT_BIN = 128;    // threads per CTA for binning (BIN_CHUNK atoms per CTA)
 constexpr int NT_SLAB = SLAB_THREADS;  // threads per CTA for the forward / inverse slab FFT stages
 constexpr int NT_TILE = 256;   // threads per CTA for spreading and force interpolation (two per atom), at most,
@@ -20,14 +21,20 @@ PME_HD int tile_nt_bound(int T) { return T >= 16 ? NT_TILE16 : NT_TILE; }
 // and twice as many CTAs fit on an SM. Dense 8^3 tiles interpolate forces on 192 threads: at 64 registers,
 // five such CTAs fit on an SM, three beside an inverse-stage CTA that has not retired yet, so all tiles of
 // a 64^3 mesh are dispatched at once (with 256 threads, 13-15 SMs ran a fifth tile in a second wave; 28.65
-// vs 28.75 us per evaluation). 16^3 tiles (hundreds of atoms each): 512 threads for spreading, 128
-// for force interpolation, whose 106 registers per thread (p = 6) leave room for four 128-thread CTAs per
-// SM but only one 512-thread CTA, so all tiles of a 128^3 mesh fit in one wave (128^3, p = 6: 131.6 vs
-// 133.6 us per evaluation with 256 threads, 145.4 with 512). Results do not depend on it.
+// vs 28.75 us per evaluation). 16^3 tiles (hundreds of atoms each) spread on 512 threads. Their force interpolation
+// takes 512 threads too where there are few tiles per SM, so that each ends soon (p = 8, 80 x 80 x 96, 150 tiles: 73 us
+// per evaluation against 88 with 256 or 128 threads); 256 at orders 5 and 6 with few atoms a tile, whose 512 threads
+// would idle (90 x 96 x 100, 25000 atoms, p = 6: 53 against 58 with 512); and 128 where more than three tiles per SM at
+// orders 6 and 8 would come in waves (106 registers at p = 6: four 128-thread CTAs per SM but only one of 512;
+// 128^3, 262144 atoms, p = 6: 126 against 129 with 256 and 131 with 512). Results do not depend on it.
 inline int tile_threads(const SysDev &d, int64_t n, bool gather = false) {
     if (d.nt_tile == 128 || d.nt_tile == NT_TILE || (d.nt_tile == NT_TILE16 && d.tlog >= 4))
         return d.nt_tile;  // chosen by the autotuner or the caller
-    if (d.tlog >= 4) return gather ? 128 : NT_TILE16;
+    if (d.tlog >= 4) {
+        if (!gather) return NT_TILE16;
+        if (d.p >= 6 && d.ntiles > 3 * GB300_SMS) return 128;
+        return (d.p == 5 || d.p == 6) && n < (int64_t)200 * d.ntiles ? 256 : NT_TILE16;
+    }
     if (d.ntiles > 0 && n <= (int64_t)64 * d.ntiles) return 128;
     return gather ? 192 : NT_TILE;
 }

@@ -156,7 +156,7 @@ pme_status plan_reserve(pme_plan *pl, int64_t n) {
     const int64_t ncap = n > 0 ? n : 1;
     // tile edge from the atom density, or the one the autotuner / caller set (every tile counter is zero
     // between evaluations, so the tiling may change here; results do not depend on it)
-    set_tiling(d, pl->tile_log_set ? pl->tile_log_set : choose_tile_log(ncap, pl->K, pl->sms));
+    set_tiling(d, pl->tile_log_set ? pl->tile_log_set : choose_tile_log(ncap, pl->K, pl->sms, pl->p));
     set_tiling(d, d.tlog, choose_k1_pieces(d, pl->sms));
     const int cap = bucket_capacity(ncap, d.ntiles, d.tlog);
     const size_t nb = (size_t)d.ntiles * cap;

@@ -291,7 +291,7 @@ pme_status pme_autotune(pme_plan *pl, const float *pos, const float *q, int64_t 
         return PME_OK;
     }
     // candidates: the default first (its results are the reference bits), then every other combination
-    const int tdef = pl->tile_log_set ? pl->tile_log_set : choose_tile_log(n > 0 ? n : 1, pl->K, pl->sms);
+    const int tdef = pl->tile_log_set ? pl->tile_log_set : choose_tile_log(n > 0 ? n : 1, pl->K, pl->sms, pl->p);
     if ((st = plan_retile(pl, tdef, 0, n)) != PME_OK) return st;
     // the default sizes (nt = 0): spreading and force interpolation take different CTA sizes
     const int ntdef = 0;

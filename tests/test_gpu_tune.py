@@ -67,6 +67,32 @@ def test_every_tiling_candidate_is_bit_identical(pme, oracle_mod, name):
         pme.pme_destroy(plan)
 
 
+# mesh, order, atoms, the default tile edge on 152 SMs: either side of the tile-count and density lines
+DEFAULT_EDGES = [((80, 80, 96), 6, 5000, 16), ((80, 80, 80), 6, 5000, 8), ((80, 80, 96), 4, 6000, 8), ((72, 80, 100), 4, 6000, 16),
+                 ((80, 80, 96), 8, 4000, 8), ((80, 80, 100), 5, 60000, 16), ((128, 128, 128), 8, 17000, 16)]
+
+
+@pytest.mark.parametrize("K,p,n,edge", DEFAULT_EDGES, ids=[f"{K[0]}x{K[1]}x{K[2]}_p{p}_{n}" for K, p, n, _ in DEFAULT_EDGES])
+def test_default_tile_edge(pme, K, p, n, edge):
+    """The default edge, and the other edge's energy, virial and forces equal to its own bit for bit."""
+    L = np.array(K, dtype=float) * 1.1
+    rng = np.random.default_rng(n)
+    P = torch.from_numpy((rng.random((n, 3)) * L).astype(np.float32)).cuda()
+    q = rng.normal(size=n)
+    Q = torch.from_numpy((q - q.mean()).astype(np.float32)).cuda()
+    plan = pme.pme_create(K, p, 0.34, np.diag(L))
+    try:
+        F0, F = torch.empty_like(P), torch.empty_like(P)
+        E0, V0 = pme.pme_compute(plan, P, Q, F0)
+        if torch.cuda.get_device_properties(0).multi_processor_count == 152:
+            assert pme.pme_plan_get_tiling(plan) == (edge, 0)
+        pme.pme_plan_set_tiling(plan, 24 - edge, 0)
+        E, V = pme.pme_compute(plan, P, Q, F)
+        assert E == E0 and np.array_equal(V, V0) and torch.equal(F, F0)
+    finally:
+        pme.pme_destroy(plan)
+
+
 def test_autotune_picks_and_persists(pme, tmp_path):
     s = wl.headline_system()
     P, Q = _dev(s)
