@@ -16,16 +16,15 @@ namespace pme {
 
 constexpr int MD_CHUNK = 32;   // steps per recorded graph
 constexpr int MD_EV = 15;      // doubles per step in ev_steps: E_rec, virial_rec[6], E_real, E_self, virial_real[6]
-constexpr size_t MD_MEM = 256; // counter (16 B) + real-space energies (8 doubles), padded
+constexpr size_t MD_MEM = 256; // step counters of the update and of the real-space energies, 128 bytes apart
 
 struct LeapArgs {
-    float *pos, *vel;
-    const float *forces, *inv_mass;
+    float *pos, *vel, *forces;  // forces: the reciprocal part, replaced by the sum where there is a real part
+    const float *real, *inv_mass;  // real-space part or null; null: unit mass
     int n;
     float dt;
     const double *ev_rec;   // the plan's energy / virial of this step (7 doubles)
-    const double *ev_real;  // the real-space energies of this step (8 doubles) or null
-    double *ev_steps;       // steps x MD_EV or null
+    double *ev_steps;       // steps x MD_EV or null (the real-space columns are filed by its own reduction)
     unsigned *counter;      // steps completed in this call
     int steps;
 };
@@ -40,7 +39,12 @@ __global__ void __launch_bounds__(256) k_leapfrog(LeapArgs a) {
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             const size_t j = 3 * (size_t)i + k;
-            const float v = __fadd_rn(a.vel[j], __fmul_rn(__fmul_rn(a.forces[j], im), a.dt));
+            float f = a.forces[j];
+            if (a.real) {
+                f = __fadd_rn(f, a.real[j]);
+                a.forces[j] = f;
+            }
+            const float v = __fadd_rn(a.vel[j], __fmul_rn(__fmul_rn(f, im), a.dt));
             a.vel[j] = v;
             a.pos[j] = __fadd_rn(a.pos[j], __fmul_rn(v, a.dt));
         }
@@ -49,12 +53,9 @@ __global__ void __launch_bounds__(256) k_leapfrog(LeapArgs a) {
         __shared__ unsigned step;
         if (threadIdx.x == 0) step = *a.counter;
         __syncthreads();
-        if (a.ev_steps && step < (unsigned)a.steps && threadIdx.x < MD_EV) {
+        if (a.ev_steps && step < (unsigned)a.steps && threadIdx.x < (a.real ? 7 : MD_EV)) {
             const int t = threadIdx.x;
-            double v = 0.0;
-            if (t < 7) v = a.ev_rec[t];
-            else if (a.ev_real) v = a.ev_real[t - 7];
-            a.ev_steps[(size_t)step * MD_EV + t] = v;
+            a.ev_steps[(size_t)step * MD_EV + t] = t < 7 ? a.ev_rec[t] : 0.0;
         }
         __syncthreads();
         if (threadIdx.x == 0) *a.counter = step + 1u;
@@ -90,29 +91,56 @@ extern "C" pme_status pme_run_steps(pme_plan *pl, pme_real *rs, float *pos, floa
         }
     }
     if (steps == 0) return PME_OK;
-    unsigned *counter = (unsigned *)pl->md_mem;
-    double *ev_real = (double *)((char *)pl->md_mem + 16);
+    unsigned *counter = (unsigned *)pl->md_mem, *real_counter = counter + 32;
     if ((e = cudaMemsetAsync(pl->md_mem, 0, MD_MEM, pl->stream)) != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
+    if (rs && !pl->md_done) {
+        int least = 0, greatest = 0;
+        if ((e = cudaDeviceGetStreamPriorityRange(&least, &greatest)) != cudaSuccess) return cuda_fail(e, "stream priorities");
+        if ((!pl->md_main && (e = cudaStreamCreateWithPriority(&pl->md_main, cudaStreamNonBlocking, greatest)) != cudaSuccess) ||
+            (!pl->md_side && (e = cudaStreamCreateWithPriority(&pl->md_side, cudaStreamNonBlocking, least)) != cudaSuccess))
+            return cuda_fail(e, "cudaStreamCreate");
+        for (cudaEvent_t *ev : {&pl->md_fork, &pl->md_pairs, &pl->md_done})
+            if (!*ev && (e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming)) != cudaSuccess) {
+                *ev = nullptr;
+                return cuda_fail(e, "cudaEventCreate");
+            }
+    }
 
     const SysDev d = plan_descriptor(pl, pos, q, n, forces, nullptr);
     LeapArgs la;
     la.pos = pos;
     la.vel = vel;
     la.forces = forces;
+    la.real = nullptr;
     la.inv_mass = inv_mass;
     la.n = (int)n;
     la.dt = (float)dt;
     la.ev_rec = pl->d.ctl->ev;
-    la.ev_real = rs ? ev_real : nullptr;
     la.ev_steps = ev_steps;
     la.counter = counter;
     la.steps = steps;
-    // one step: reciprocal forces (written), real-space forces (added), the update
+    // One step on stream s: reciprocal forces, then the update. With real space, its kernels run beside the
+    // reciprocal stages on the side stream into an array of their own, and the update adds the two parts (the same
+    // sums as one after the other); the real-space energies are reduced beside the update. The stages leave most
+    // of the GPU idle (six latency chains), and the pair kernel fills it: 8190 atoms, 40^3, 63 -> 38 us a step.
     auto one_step = [&](cudaStream_t s) -> cudaError_t {
-        cudaError_t r = launch_pipeline(d, s);
-        if (r != cudaSuccess) return r;
-        if (rs && real_enqueue_on(rs, s, pos, q, n, forces, 1, ev_real) != PME_OK) return cudaErrorLaunchFailure;
+        cudaError_t r;
+        if (rs) {
+            if ((r = cudaEventRecord(pl->md_fork, s)) != cudaSuccess || (r = cudaStreamWaitEvent(pl->md_side, pl->md_fork, 0)) != cudaSuccess)
+                return r;
+            la.real = real_enqueue_own(rs, pl->md_side, pos, q, n);
+            if ((r = cudaEventRecord(pl->md_pairs, pl->md_side)) != cudaSuccess) return r;
+            real_enqueue_file(rs, pl->md_side, n, real_counter, ev_steps ? ev_steps + 7 : nullptr, MD_EV, steps);
+        }
+        if ((r = launch_pipeline(d, s)) != cudaSuccess) return r;
+        if (rs && (r = cudaStreamWaitEvent(s, pl->md_pairs, 0)) != cudaSuccess) return r;
         return launch_leapfrog(la, s);
+    };
+    // the side stream's last work back into s
+    auto join = [&](cudaStream_t s) -> cudaError_t {
+        if (!rs) return cudaSuccess;
+        const cudaError_t r = cudaEventRecord(pl->md_done, pl->md_side);
+        return r != cudaSuccess ? r : cudaStreamWaitEvent(s, pl->md_done, 0);
     };
     const int chunk = steps < MD_CHUNK ? steps : MD_CHUNK;
     pme_plan::StepGraph key;
@@ -140,12 +168,14 @@ extern "C" pme_status pme_run_steps(pme_plan *pl, pme_real *rs, float *pos, floa
         gm = pme_plan::StepGraph();
         if (!pl->rec_stream && (e = cudaStreamCreateWithFlags(&pl->rec_stream, cudaStreamNonBlocking)) != cudaSuccess)
             return cuda_fail(e, "cudaStreamCreate");
-        if ((e = cudaStreamBeginCapture(pl->rec_stream, cudaStreamCaptureModeThreadLocal)) != cudaSuccess)
+        const cudaStream_t rec = rs ? pl->md_main : pl->rec_stream;
+        if ((e = cudaStreamBeginCapture(rec, cudaStreamCaptureModeThreadLocal)) != cudaSuccess)
             return cuda_fail(e, "cudaStreamBeginCapture");
         cudaError_t r = cudaSuccess;
-        for (int i = 0; i < chunk && r == cudaSuccess; ++i) r = one_step(pl->rec_stream);
+        for (int i = 0; i < chunk && r == cudaSuccess; ++i) r = one_step(rec);
+        if (r == cudaSuccess) r = join(rec);
         cudaGraph_t graph = nullptr;
-        e = cudaStreamEndCapture(pl->rec_stream, &graph);
+        e = cudaStreamEndCapture(rec, &graph);
         if (r != cudaSuccess || e != cudaSuccess) {
             if (graph) cudaGraphDestroy(graph);
             return cuda_fail(r != cudaSuccess ? r : e, "recording the step loop");
@@ -161,5 +191,6 @@ extern "C" pme_status pme_run_steps(pme_plan *pl, pme_real *rs, float *pos, floa
         if ((e = cudaGraphLaunch(gm.exec, pl->stream)) != cudaSuccess) return cuda_fail(e, "cudaGraphLaunch(step loop)");
     for (int i = steps - steps % chunk; i < steps; ++i)  // the remainder, launched directly
         if ((e = one_step(pl->stream)) != cudaSuccess) return cuda_fail(e, "step launch");
+    if (steps % chunk && (e = join(pl->stream)) != cudaSuccess) return cuda_fail(e, "step launch");
     return PME_OK;
 }

@@ -769,11 +769,13 @@ void pme_destroy(pme_plan *pl) {
     if (pl->md_mem) cudaFree(pl->md_mem);
     if (pl->tc_w) cudaFree(pl->tc_w);
     if (pl->rec_stream) cudaStreamDestroy(pl->rec_stream);
-    for (cudaStream_t cs : {pl->copy_stream, pl->out_stream})
+    for (cudaStream_t cs : {pl->copy_stream, pl->out_stream, pl->md_side, pl->md_main})
         if (cs) {
             cudaStreamSynchronize(cs);
             cudaStreamDestroy(cs);
         }
+    for (cudaEvent_t ev : {pl->md_fork, pl->md_pairs, pl->md_done})
+        if (ev) cudaEventDestroy(ev);
     for (int s = 0; s < 2; ++s)
         for (cudaEvent_t ev : {pl->in_ready[s], pl->in_free[s], pl->out_done[s]})
             if (ev) cudaEventDestroy(ev);

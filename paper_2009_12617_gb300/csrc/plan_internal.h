@@ -64,9 +64,13 @@ struct pme_plan {
     cudaEvent_t host_done[HOST_TICKETS] = {};
     int64_t host_seq = 0;
     cudaStream_t rec_stream = nullptr;
-    // multi-step loop (pme_run_steps): step counter and real-space energies, and the recorded graph of one
+    // multi-step loop (pme_run_steps): step counters, and the recorded graph of one
     // chunk of steps for the last argument set
     void *md_mem = nullptr;
+    // with real space: the streams its steps are recorded on (the reciprocal stages on md_main, of higher priority, the
+    // real-space kernels beside them on md_side), and the events between them
+    cudaStream_t md_main = nullptr, md_side = nullptr;
+    cudaEvent_t md_fork = nullptr, md_pairs = nullptr, md_done = nullptr;
     struct StepGraph {
         cudaGraphExec_t exec = nullptr;
         const void *pos = nullptr, *vel = nullptr, *q = nullptr, *inv_mass = nullptr, *forces = nullptr,
@@ -104,6 +108,8 @@ pme_status plan_retile(pme_plan *pl, int tlog, int nt, int64_t n);
 pme_status real_enqueue_on(pme_real *rs, cudaStream_t stream, const float *pos, const float *q, int64_t n,
                            float *forces, int accumulate, double *ev_dev);
 pme_status real_reserve_n(pme_real *rs, int64_t n);
+const float *real_enqueue_own(pme_real *rs, cudaStream_t stream, const float *pos, const float *q, int64_t n);
+void real_enqueue_file(pme_real *rs, cudaStream_t stream, int64_t n, unsigned *step, double *file, int stride, int rows);
 int real_device(const pme_real *rs);
 unsigned long long real_gen(const pme_real *rs);  // changes whenever a recorded launch of rs would be stale
 SysDev plan_descriptor(const pme_plan *pl, const float *pos, const float *q, int64_t n, float *forces, double *ev_dev);

@@ -33,11 +33,11 @@ namespace pme {
 
 constexpr int RS_SCAN_THREADS = 1024;
 constexpr int RS_BIN_THREADS = 256;
-constexpr int RS_RED_BLOCKS = 64;   // level-one blocks of the final reduction
+constexpr int RS_RED_BLOCKS = 16;   // level-one blocks of the final reduction
 constexpr int RS_MAX_R = 4;         // cutoffs of up to 4 cell widths per axis (cells at least a cutoff wide)
 constexpr int RS_MAX_CELLS = 1 << 22;
 constexpr int RS_CAND = 192;        // candidates a warp of the pair kernel holds at a time
-constexpr int RS_SUMS = 7;          // energy, virial xx yy zz xy xz yz
+constexpr int RS_SUMS = 8;          // energy, virial xx yy zz xy xz yz, q^2
 
 struct RealCtl {
     unsigned status;  // StatusBits
@@ -52,7 +52,6 @@ struct RealDev {
     int nc[3], R[3], ncells;
     int slab, nslab, nrowslabs;  // cells along axis 2 per work-item slab, slabs per row, rows x slabs
     int max_items;         // launched pair CTAs: n / 32 + one per occupied row slab, at most
-    int q_blocks;          // binning CTAs (partial sums of q^2)
     float rec[9];          // a*_alpha[j] at 3 alpha + j (cell assignment)
     int afix[9];           // a_alpha[k] / u at 3 alpha + k, low 32 bits of the nearest integer
     float afrac[9];        // what is left of a_alpha[k] / u, in [-1/2, 1/2]
@@ -65,6 +64,11 @@ struct RealDev {
     const float *pos, *q;
     float *forces;
     double *ev;            // optional device destination of RealCtl::res (8 doubles)
+    // optional: step number file_step[0] (advanced here) and a row of file_stride doubles per step, to hold
+    // RealCtl::res for steps below file_rows
+    unsigned *file_step;
+    double *file;
+    int file_stride, file_rows;
     unsigned *count;       // ncells, zero between calls (reset by the scan)
     unsigned *start;       // ncells + 1
     int2 *cell;            // n: input atom i's cell and arrival number in it
@@ -74,8 +78,8 @@ struct RealDev {
     int *sidx;             // n: input index likewise
     int *scell;            // n: cell likewise
     int2 *items;           // first sorted atom and atom count of each work item
-    double *q2;            // q_blocks: sums of q^2
-    double *sums;          // 8 per work item: energy and virial sums of each work item
+    double *sums;          // RS_SUMS per work item
+    float *fown;           // 3 n: forces of real_enqueue_own
     double *partials;      // RS_RED_BLOCKS x 8
     RealCtl *ctl;
 };
@@ -92,32 +96,11 @@ __device__ __forceinline__ int image_offset(const RealDev &d, int k, int m0, int
 
 __device__ __forceinline__ int floordiv(int a, int b) { return a >= 0 ? a / b : -((-a + b - 1) / b); }
 
-// FP64 block sum of NV values per thread in a fixed tree (warp shuffles, then the warps' results in order).
-template <int NV>
-__device__ void block_sum(double (&v)[NV], double *out) {
-    __shared__ double wsum[NV][32];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
-        if (lane == 0) wsum[k][warp] = v[k];
-    }
-    __syncthreads();
-    if (threadIdx.x < NV) {
-        double s = 0.0;
-        for (int w = 0; w < nw; ++w) s += wsum[threadIdx.x][w];
-        out[threadIdx.x] = s;
-    }
-}
-
 // 1: per atom its cell and arrival number, and its fixed-point position: x / u rounded to an integer (exact
-// wherever x's own spacing is at least u), less the whole cells it lies out, both modulo 2^32. Per CTA the
-// sum of q^2.
+// wherever x's own spacing is at least u), less the whole cells it lies out, both modulo 2^32.
 __global__ void __launch_bounds__(RS_BIN_THREADS) k_rs_bin(RealDev d) {
     pdl_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    double q2[1] = {0.0};
     if (i < d.n) {
         const float r[3] = {d.pos[3 * (size_t)i], d.pos[3 * (size_t)i + 1], d.pos[3 * (size_t)i + 2]};
         const float qq = d.q[i];
@@ -145,9 +128,7 @@ __global__ void __launch_bounds__(RS_BIN_THREADS) k_rs_bin(RealDev d) {
         const int cid = (c[0] * d.nc[1] + c[1]) * d.nc[2] + c[2];
         d.xq[i] = make_int4(X[0], X[1], X[2], __float_as_int(qq));
         d.cell[i] = make_int2(cid, (int)atomicAdd(d.count + cid, 1u));
-        q2[0] = (double)qq * (double)qq;
     }
-    block_sum(q2, d.q2 + blockIdx.x);
 }
 
 // Exclusive scan of one value per thread over the CTA; total receives the sum. Uses warp shuffles and one
@@ -611,6 +592,14 @@ __global__ void __launch_bounds__(32 * NW, 20 / NW) k_rs_pairs(RealDev d) {
         }
     }
     for (int k = warp; k < RS_SUMS; k += NW) {
+        if (k == 7) {  // the self term, in FP64
+            double t = mine ? (double)__int_as_float(me.w) : 0.0;
+            t *= t;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+            if (lane == 0) d.sums[RS_SUMS * (size_t)blockIdx.x + k] = t;
+            continue;
+        }
         DF t = {0.f, 0.f};
 #pragma unroll
         for (int v = 0; v < NW; ++v) {
@@ -626,51 +615,62 @@ __global__ void __launch_bounds__(32 * NW, 20 / NW) k_rs_pairs(RealDev d) {
             a.lo = __shfl_down_sync(0xffffffffu, t.lo, o);
             t = df_add(t, a);
         }
-        if (lane == 0) d.sums[8 * (size_t)blockIdx.x + k] = (double)t.hi + (double)t.lo;
+        if (lane == 0) d.sums[RS_SUMS * (size_t)blockIdx.x + k] = (double)t.hi + (double)t.lo;
     }
 }
 
-// 6: the work items' sums and the binning CTAs' sums of q^2, in contiguous chunks per block; the block that
-// finishes last adds the blocks' sums in order and stores energies, self term and virial in the control block
-// (and in d.ev).
+// FP64 sums of rows of RS_SUMS values, 256 threads: thread t adds value t mod 8 of the rows [b, e) from b + t / 8 in
+// steps of 32, then the 32 partial sums meet in a fixed tree; out[k] (shared or global) by threads k < 8.
+__device__ __forceinline__ void sum_rows(const double *rows, int b, int e, double *out) {
+    __shared__ double wsum[8][RS_SUMS];
+    const int tid = threadIdx.x, k = tid & 7;
+    double v = 0.0;
+    for (int a = b + (tid >> 3); a < e; a += 32) v += __ldcg(rows + RS_SUMS * (size_t)a + k);
+    v += __shfl_down_sync(0xffffffffu, v, 16);
+    v += __shfl_down_sync(0xffffffffu, v, 8);
+    if ((tid & 31) < 8) wsum[tid >> 5][k] = v;
+    __syncthreads();
+    if (tid < 8) {
+        double s = 0.0;
+        for (int w = 0; w < 8; ++w) s += wsum[w][tid];
+        out[tid] = s;
+    }
+    __syncthreads();
+}
+
+// 6: the work items' sums, in contiguous chunks per block; the block that finishes last adds the blocks' sums in
+// order and stores energies, self term and virial in the control block, in d.ev and in d.file. Eight threads
+// share a row, one value each, since FP64 additions are slow (a thread per row with all values took 12 us at 2300
+// items).
 __global__ void __launch_bounds__(256) k_rs_reduce(RealDev d) {
     __shared__ bool last;
-    __shared__ double tot[8];
+    __shared__ double tot[RS_SUMS];
     pdl_wait();
-    const int nitems = d.n > 0 ? (int)d.ctl->nitems : 0;
-    double v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    {
-        const int chunk = (nitems + gridDim.x - 1) / gridDim.x, b = blockIdx.x * chunk, e = min(nitems, b + chunk);
-        for (int a = b + (int)threadIdx.x; a < e; a += blockDim.x)
-#pragma unroll
-            for (int k = 0; k < RS_SUMS; ++k) v[k] += d.sums[8 * (size_t)a + k];
-    }
-    {
-        const int chunk = (d.q_blocks + gridDim.x - 1) / gridDim.x, b = blockIdx.x * chunk, e = min(d.q_blocks, b + chunk);
-        for (int a = b + (int)threadIdx.x; a < e; a += blockDim.x) v[7] += d.q2[a];
-    }
-    block_sum(v, d.partials + 8 * blockIdx.x);
+    const int tid = threadIdx.x, nitems = d.n > 0 ? (int)d.ctl->nitems : 0;
+    const int chunk = (nitems + gridDim.x - 1) / gridDim.x, b = blockIdx.x * chunk;
+    sum_rows(d.sums, b, min(nitems, b + chunk), d.partials + RS_SUMS * blockIdx.x);
     __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) last = atomicAdd(&d.ctl->arrived, 1u) == gridDim.x - 1u;
+    if (tid == 0) last = atomicAdd(&d.ctl->arrived, 1u) == gridDim.x - 1u;
     __syncthreads();
     if (!last) return;
     __threadfence();
-#pragma unroll
-    for (int k = 0; k < 8; ++k) v[k] = threadIdx.x < gridDim.x ? __ldcg(d.partials + 8 * threadIdx.x + k) : 0.0;
-    block_sum(v, tot);
-    __syncthreads();
-    if (threadIdx.x == 0) {
+    sum_rows(d.partials, 0, (int)gridDim.x, tot);
+    if (tid < 8) {
+        // E_real, E_self, virial
         const double sqrt_pi = 1.7724538509055160273;
-        double r[8];
-        r[0] = 0.5 * tot[0] * d.inv_u;
-        r[1] = -d.beta_d / sqrt_pi * tot[7];
-        for (int k = 0; k < 6; ++k) r[2 + k] = 0.5 * tot[1 + k] * d.inv_u;
-        for (int k = 0; k < 8; ++k) d.ctl->res[k] = r[k];
-        if (d.ev)
-            for (int k = 0; k < 8; ++k) d.ev[k] = r[k];
-        d.ctl->arrived = 0u;
+        const double r = tid == 0 ? 0.5 * tot[0] * d.inv_u
+                                  : (tid == 1 ? -d.beta_d / sqrt_pi * tot[7] : 0.5 * tot[tid - 1] * d.inv_u);
+        d.ctl->res[tid] = r;
+        if (d.ev) d.ev[tid] = r;
+        if (d.file_step) {
+            const unsigned step = *d.file_step;
+            if (d.file && step < (unsigned)d.file_rows) d.file[(size_t)step * d.file_stride + tid] = r;
+            __syncwarp(0xffu);
+            if (tid == 0) *d.file_step = step + 1u;
+        }
     }
+    if (tid == 0) d.ctl->arrived = 0u;
 }
 
 }  // namespace pme
@@ -779,7 +779,7 @@ static pme_status real_alloc_cells(pme_real *rs) {
     size_t off = 0;
     const size_t o_cnt = off;  off = al256r(off + nc * 4);
     const size_t o_st = off;   off = al256r(off + (nc + 1) * 4);
-    const size_t o_par = off;  off = al256r(off + RS_RED_BLOCKS * 8 * sizeof(double));
+    const size_t o_par = off;  off = al256r(off + RS_RED_BLOCKS * RS_SUMS * sizeof(double));
     const size_t o_ctl = off;  off = al256r(off + sizeof(RealCtl));
     if (off > rs->cell_bytes) {
         if (rs->cell_mem) cudaFree(rs->cell_mem);
@@ -814,8 +814,8 @@ static pme_status real_reserve(pme_real *rs, int64_t n) {
     const size_t o_sidx = off; off = al256r(off + m * 4);
     const size_t o_sc = off;   off = al256r(off + m * 4);
     const size_t o_it = off;   off = al256r(off + m * 8);
-    const size_t o_q2 = off;   off = al256r(off + (m / RS_BIN_THREADS + 1) * 8);
-    const size_t o_sum = off;  off = al256r(off + m * 64);
+    const size_t o_sum = off;  off = al256r(off + m * RS_SUMS * 8);
+    const size_t o_own = off;  off = al256r(off + m * 12);
     cudaError_t e = cudaStreamSynchronize(rs->stream);
     if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
     if (rs->atom_mem) cudaFree(rs->atom_mem);
@@ -835,8 +835,8 @@ static pme_status real_reserve(pme_real *rs, int64_t n) {
     d.sidx = (int *)(b + o_sidx);
     d.scell = (int *)(b + o_sc);
     d.items = (int2 *)(b + o_it);
-    d.q2 = (double *)(b + o_q2);
     d.sums = (double *)(b + o_sum);
+    d.fown = (float *)(b + o_own);
     rs->atom_bytes = off;
     rs->n_cap = (int64_t)m;
     ++rs->gen;
@@ -865,24 +865,22 @@ static void rs_launch(void (*kernel)(RealDev), unsigned grid, unsigned block, si
 // depend on the number of warps, hence on the atom count alone.
 static int rs_pair_warps(const RealDev &d) { return d.n <= 4096 ? 16 : (d.n <= 24576 ? 8 : 4); }
 
-static cudaError_t real_launch(const RealDev &d0, cudaStream_t s) {
+static void launch_pairs(const RealDev &d0, cudaStream_t s) {
     RealDev d = d0;
     const unsigned g = (unsigned)((d.n + 255) / 256);
-    d.q_blocks = (d.n + RS_BIN_THREADS - 1) / RS_BIN_THREADS;
     d.max_items = d.n / 32 + std::min(d.n, d.nrowslabs);
-    if (d.n > 0) {
-        rs_launch(k_rs_bin, (unsigned)d.q_blocks, RS_BIN_THREADS, 0, s, d);
-        rs_launch(k_rs_scan, 1, RS_SCAN_THREADS, 0, s, d);
-        rs_launch(k_rs_scatter, g, 256, 0, s, d);
-        rs_launch(k_rs_rank, g, 256, 0, s, d);
-        const int warps = rs_pair_warps(d);
-        if (warps == 4) rs_launch(k_rs_pairs<4>, (unsigned)d.max_items, 128, sizeof(RsShared<4>), s, d);
-        else if (warps == 8) rs_launch(k_rs_pairs<8>, (unsigned)d.max_items, 256, sizeof(RsShared<8>), s, d);
-        else rs_launch(k_rs_pairs<16>, (unsigned)d.max_items, 512, sizeof(RsShared<16>), s, d);
-    }
-    rs_launch(k_rs_reduce, RS_RED_BLOCKS, 256, 0, s, d);
-    return cudaGetLastError();
+    if (d.n < 1) return;
+    rs_launch(k_rs_bin, (unsigned)((d.n + RS_BIN_THREADS - 1) / RS_BIN_THREADS), RS_BIN_THREADS, 0, s, d);
+    rs_launch(k_rs_scan, 1, RS_SCAN_THREADS, 0, s, d);
+    rs_launch(k_rs_scatter, g, 256, 0, s, d);
+    rs_launch(k_rs_rank, g, 256, 0, s, d);
+    const int warps = rs_pair_warps(d);
+    if (warps == 4) rs_launch(k_rs_pairs<4>, (unsigned)d.max_items, 128, sizeof(RsShared<4>), s, d);
+    else if (warps == 8) rs_launch(k_rs_pairs<8>, (unsigned)d.max_items, 256, sizeof(RsShared<8>), s, d);
+    else rs_launch(k_rs_pairs<16>, (unsigned)d.max_items, 512, sizeof(RsShared<16>), s, d);
 }
+
+static void launch_reduce(const RealDev &d, cudaStream_t s) { rs_launch(k_rs_reduce, RS_RED_BLOCKS, 256, 0, s, d); }
 
 extern "C" {
 
@@ -977,9 +975,32 @@ pme_status pme::real_enqueue_on(pme_real *rs, cudaStream_t stream, const float *
     d.forces = forces;
     d.accumulate = accumulate ? 1 : 0;
     d.ev = ev_dev;
-    const cudaError_t e = real_launch(d, stream);
+    launch_pairs(d, stream);
+    launch_reduce(d, stream);
+    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_fail(e, "real-space kernel launch");
     return PME_OK;
+}
+
+// The evaluation into the context's own force array, in two parts: forces (the array is returned; n has been
+// reserved), then energies, filed as one row of a table per call.
+const float *pme::real_enqueue_own(pme_real *rs, cudaStream_t stream, const float *pos, const float *q, int64_t n) {
+    RealDev d = rs->d;
+    d.n = (int)n;
+    d.pos = pos;
+    d.q = q;
+    d.forces = d.fown;
+    launch_pairs(d, stream);
+    return d.fown;
+}
+void pme::real_enqueue_file(pme_real *rs, cudaStream_t stream, int64_t n, unsigned *step, double *file, int stride, int rows) {
+    RealDev d = rs->d;
+    d.n = (int)n;
+    d.file_step = step;
+    d.file = file;
+    d.file_stride = stride;
+    d.file_rows = rows;
+    launch_reduce(d, stream);
 }
 
 pme_status pme::real_reserve_n(pme_real *rs, int64_t n) {
