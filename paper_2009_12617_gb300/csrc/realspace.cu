@@ -69,6 +69,7 @@ struct RealDev {
     unsigned *file_step;
     double *file;
     int file_stride, file_rows;
+    RealCtl *host;         // optional page-locked copy of the control block's status and results (device address)
     unsigned *count;       // ncells, zero between calls (reset by the scan)
     unsigned *start;       // ncells + 1
     int2 *cell;            // n: input atom i's cell and arrival number in it
@@ -663,6 +664,10 @@ __global__ void __launch_bounds__(256) k_rs_reduce(RealDev d) {
                                   : (tid == 1 ? -d.beta_d / sqrt_pi * tot[7] : 0.5 * tot[tid - 1] * d.inv_u);
         d.ctl->res[tid] = r;
         if (d.ev) d.ev[tid] = r;
+        if (d.host) {
+            d.host->res[tid] = r;
+            if (tid == 0) d.host->status = __ldcg(&d.ctl->status);
+        }
         if (d.file_step) {
             const unsigned step = *d.file_step;
             if (d.file && step < (unsigned)d.file_rows) d.file[(size_t)step * d.file_stride + tid] = r;
@@ -687,7 +692,7 @@ struct pme_real {
     void *atom_mem = nullptr;  // per-atom scratch (grows with n)
     size_t atom_bytes = 0;
     int64_t n_cap = 0;
-    RealCtl *h_ctl = nullptr;
+    RealCtl *h_ctl = nullptr, *h_ctl_dev = nullptr;  // page-locked results of the synchronous call
     unsigned long long gen = 0;  // bumped whenever the kernels' arguments change (cell, scratch)
 };
 
@@ -922,6 +927,10 @@ pme_status pme_real_create(const double box[9], double beta, double rcut, void *
         return cuda_fail(e, "cudaMallocHost");
     }
     memset(rs->h_ctl, 0, sizeof(RealCtl));
+    if ((e = cudaHostGetDevicePointer((void **)&rs->h_ctl_dev, rs->h_ctl, 0)) != cudaSuccess) {
+        pme_real_destroy(rs);
+        return cuda_fail(e, "cudaHostGetDevicePointer");
+    }
     if ((e = cudaStreamSynchronize(rs->stream)) != cudaSuccess) {
         pme_real_destroy(rs);
         return cuda_fail(e, "cudaStreamSynchronize");
@@ -1015,12 +1024,15 @@ extern "C" {
 
 pme_status pme_real_compute(pme_real *rs, const float *pos, const float *q, int64_t n, float *forces,
                             double *e_real, double *e_self, double *virial) {
-    pme_status st = pme_real_enqueue(rs, pos, q, n, forces, 0, nullptr);
+    if (!rs) return fail(PME_EINVAL, "real-space context is NULL");
+    // the reduction stores the results and the status word in page-locked memory itself (a copy-engine transfer
+    // of the block after it took 7 us more: 2048 atoms, 52 -> 45 us)
+    rs->d.host = rs->h_ctl_dev;
+    pme_status st = real_enqueue_on(rs, rs->stream, pos, q, n, forces, 0, nullptr);
+    rs->d.host = nullptr;
     if (st != PME_OK) return st;
     DeviceGuard g(rs->dev);
     cudaError_t e;
-    if ((e = cudaMemcpyAsync(rs->h_ctl, rs->d.ctl, sizeof(RealCtl), cudaMemcpyDeviceToHost, rs->stream)) != cudaSuccess)
-        return cuda_fail(e, "cudaMemcpyAsync(result)");
     if ((e = cudaStreamSynchronize(rs->stream)) != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
     const unsigned bits = rs->h_ctl->status;
     if (bits) {
