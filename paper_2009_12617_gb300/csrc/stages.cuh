@@ -103,17 +103,29 @@ struct SpreadLayout {
 // shared-memory sizes (bytes) of each stage for a given system and block size
 
 inline size_t smem_bin(int nth) { return (size_t)((nth + 31) / 32) * sizeof(unsigned long long) + 16; }
-inline size_t smem_tile_region(int p, int tlog) {
-    const size_t r = (size_t)(1 << tlog) + p - 1;
-    return r * r * r;
-}
 // split accumulators over the padded region (2 x spread_vol ints), cap = cap_max_for(tlog) records of
 // spread_rec_bytes and 16 residue counters
 inline size_t smem_spread(int p, int tlog) {
     return (size_t)2 * spread_vol(p, tlog) * sizeof(int) + (size_t)cap_max_for(tlog) * spread_rec_bytes(p, tlog) +
            16 * sizeof(unsigned);
 }
-inline size_t smem_gather(int p, int tlog) { return smem_tile_region(p, tlog) * sizeof(float); }
+// Whether spreading leaves its buckets in dealt order for the force stage, whose reads of the potential then fall on
+// distinct banks like the spreading's additions: 16^3 tiles from order 5. It costs writing the records back and pays
+// with many points per atom (force stage, us: 128^3, 262144 atoms, p = 6 39.5 -> 35.2, p = 8 68.7 -> 55.2; evaluations
+// 126 -> 123, 198 -> 184; 90 x 96 x 100, p = 8 93 -> 88); with 8^3 tiles (64^3, p = 6 42.2 -> 43.2) and at p = 4 (128^3
+// 90.2 -> 91.7) it does not, nor with few atoms in a tile (90 x 96 x 100, 25000 atoms, p = 6 56.7 -> 57.2 without
+// the limit of DEALT_MIN).
+constexpr int DEALT_MIN = 256;
+PME_HD bool dealt_buckets(int p, int tlog) { return tlog >= 4 && p >= 5; }
+// Region of the potential in the force stage: rows R apart, planes as far apart as the spreading region's where
+// the bucket is in dealt order (an atom's two half-support lanes 16 banks apart, see spread_plane), else R^2.
+PME_HD int gather_plane(int p, int tlog) {
+    const int R = (1 << tlog) + p - 1;
+    return dealt_buckets(p, tlog) ? spread_plane(p, tlog) : R * R;
+}
+inline size_t smem_gather(int p, int tlog) {
+    return (size_t)((1 << tlog) + p - 1) * gather_plane(p, tlog) * sizeof(float);
+}
 // Two K2 x H3 buffers (the register path uses one, with rows padded by up to 15), then the twiddles.
 inline size_t smem_slab(int K2, int K3) {
     const int H3 = K3 / 2 + 1;
@@ -492,8 +504,8 @@ PME_DEV void stage_spread(const SysDev &d, int item, void *smem, bool cleared = 
     } else {
         tile_origin(d, item, o1, o2, o3);
     }
-    const float4 *A = d.bka + (size_t)item * d.cap;
-    const int2 *B = d.bkb + (size_t)item * d.cap;
+    float4 *A = d.bka + (size_t)item * d.cap;
+    int2 *B = d.bkb + (size_t)item * d.cap;
     // this thread's first record in flight with the count, for the threads below the mean occupancy (the
     // bucket capacity is twice it plus a margin), so that few loads land on empty slots
     const bool pf = tid < (d.cap >> 1);
@@ -574,6 +586,12 @@ PME_DEV void stage_spread(const SysDev &d, int item, void *smem, bool cleared = 
             }
         }
         PME_SYNC();
+        if (dealt_buckets(P, SpreadLayout<P, T>::TLOG) && cnt >= DEALT_MIN) {
+            for (int pos = tid; pos < cnt; pos += nth) {
+                A[pos] = ra_s[inv_s[pos]];
+                B[pos] = rb_s[inv_s[pos]];
+            }
+        }
         // two threads per atom: half 0 takes the planes j1 in [0, H0), half 1 [H0, P)
         constexpr int H0 = half_planes(P);
         for (int a2 = tid; a2 < 2 * cnt; a2 += nth) {
@@ -1586,7 +1604,7 @@ PME_DEV void stage_gather(const SysDev &d, int item, void *smem, const int *org 
         for (unsigned a = (unsigned)((item - d.ntiles) * nth + tid); a < novf; a += (unsigned)(OVF_ITEMS * nth))
             gather_atom_global<P>(d, ldcg(d.ova + a), ldcg(d.ovb + a));
     } else {
-        constexpr int R = Region<P, T>::R, H = P - 1;
+        constexpr int R = Region<P, T>::R, H = P - 1, PL = gather_plane(P, T >= 16 ? 4 : 3);
         float *reg = (float *)smem;
         int o1, o2, o3;
         if (org) {
@@ -1623,15 +1641,17 @@ PME_DEV void stage_gather(const SysDev &d, int item, void *smem, const int *org 
                         }
                     }
 #pragma unroll
-                    for (int u = 0; u < LOAD_BATCH; ++u)
-                        if (r0 + u * ng < R1 * R) reg[(r0 + u * ng) * R + i3] = v[u];
+                    for (int u = 0; u < LOAD_BATCH; ++u) {
+                        const int r = r0 + u * ng;
+                        if (r < R1 * R) reg[r * R + (r / R) * (PL - R * R) + i3] = v[u];
+                    }
                 }
             }
         } else {
             for (int i = tid; i < R1 * R * R; i += nth) {
                 const int i3 = i % R, i2 = (i / R) % R, i1 = i / (R * R);
                 const int k1 = wrapk(o1 - H + i1, d.K1), k2 = wrapk(o2 - H + i2, d.K2), k3 = wrapk(o3 - H + i3, d.K3);
-                reg[i] = ldcg(d.phi + ((size_t)k1 * d.K2 + k2) * d.K3 + k3);
+                reg[i1 * PL + i2 * R + i3] = ldcg(d.phi + ((size_t)k1 * d.K2 + k2) * d.K3 + k3);
             }
         }
         PME_SYNC();
@@ -1664,7 +1684,7 @@ PME_DEV void stage_gather(const SysDev &d, int item, void *smem, const int *org 
                 const float dt1 = half ? dth1[jh] : dth1[jj];
 #pragma unroll
                 for (int j2 = 0; j2 < P; ++j2) {
-                    const float *row = reg + ((l1 - j1) * R + (l2 - j2)) * R + l3;
+                    const float *row = reg + (l1 - j1) * PL + (l2 - j2) * R + l3;
                     float s = 0.f, ds = 0.f;
 #pragma unroll
                     for (int j3 = 0; j3 < P; ++j3) {
