@@ -865,10 +865,12 @@ static void rs_launch(void (*kernel)(RealDev), unsigned grid, unsigned block, si
 
 // Warps per work item. An item needs about 28 atoms' worth of a CTA, so small systems have few CTAs and gain
 // from more warps in each; large ones fill the GPU with either and evaluate with fewer idle lanes when a warp
-// sees more of the candidates. Measured with 4 / 8 / 16 warps (us): real space of 2048 atoms 66 / 58 / 54; 32
-// MD steps of 8190 atoms 2338 / 2019 / 2180; full Ewald of 65536 atoms 169 / 193 / 235. The sums of a system
-// depend on the number of warps, hence on the atom count alone.
-static int rs_pair_warps(const RealDev &d) { return d.n <= 4096 ? 16 : (d.n <= 24576 ? 8 : 4); }
+// sees more of the candidates. Measured with 4 / 8 / 16 warps (us): real space of 2048 atoms 66 / 58 / 54, of 3500
+// - / 50 / 45, of 18000 76 / 82 / -; 32 MD steps of 8190 atoms 2338 / 2019 / 2180, of 12000 1866 / 1692 / -, of 18000
+// 1952 / 2102 / -; full Ewald of 65536 atoms 169 / 193 / 235. (Six warps, three CTAs per SM, for 300 to 456 items: 32
+// steps of 8190 atoms 1424 against 1199 with eight.) A system's sums depend on the number of warps, hence on the atom
+// count alone.
+static int rs_pair_warps(const RealDev &d) { return d.n <= 4096 ? 16 : (d.n <= 15000 ? 8 : 4); }
 
 static void launch_pairs(const RealDev &d0, cudaStream_t s) {
     RealDev d = d0;

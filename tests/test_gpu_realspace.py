@@ -183,7 +183,7 @@ EDGES = {
     "skewed": (1200, np.array([[24.0, 0, 0], [11.0, 22.0, 0], [-10.0, 9.0, 25.0]]), 8.0),
     "dense": (3000, np.eye(3) * 16.0, 6.0),                # hits of every candidate block, full rings
     "eight_warps": (4099, np.eye(3) * 34.5, 5.0),
-    "four_warps": (24580, np.eye(3) * 62.7, 3.0),
+    "four_warps": (15010, np.eye(3) * 53.2, 4.0),
 }
 
 
