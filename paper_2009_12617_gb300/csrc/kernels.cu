@@ -11,7 +11,9 @@ namespace pme {
 static int g_launch_mode = 2;  // measured fastest on GB300 (late trigger)
 void set_launch_mode(int mode) { g_launch_mode = mode; }
 int launch_mode() { return g_launch_mode; }
-int pdl_when(int mode, int stage) { return mode == 1 ? 0 : (mode == 3 || stage == STAGE_CONV ? 2 : 1); }
+int pdl_when(int mode, int stage, const SysDev &d) {
+    return mode == 1 ? 0 : (mode == 3 || (stage == STAGE_CONV && d.K1 <= 64) ? 2 : 1);
+}
 
 __global__ void __launch_bounds__(NT_BIN) k_bin(SysDev d) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -72,7 +74,7 @@ __global__ void __launch_bounds__(tile_nt_bound(T)) k_gather(SysDev d) {
 static void launch_pdl(void (*kernel)(SysDev), unsigned grid, unsigned block, size_t smem, cudaStream_t s,
                        const SysDev &d0, int stage, unsigned cluster = 1) {
     SysDev d = d0;
-    d.pdl_late = pdl_when(g_launch_mode, stage);
+    d.pdl_late = pdl_when(g_launch_mode, stage, d0);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(block);
@@ -119,11 +121,9 @@ static bool launch_split_slab(const SysDev &d, bool fwd, int count, cudaStream_t
 #define PME_SPLIT_LAUNCH(K, CS)                                                                                  \
     if (d.K2 == K && cs == CS) {                                                                                 \
         if (fwd)                                                                                                 \
-            launch_pdl(k_fwd_c<K, CS>, (unsigned)(count * CS), SlabSplit<K, CS>::NT_FWD, smem_slab(K, K), s, d, \
-                       STAGE_FWD, CS);                                                                           \
+            launch_pdl(k_fwd_c<K, CS>, (unsigned)(count * CS), SlabSplit<K, CS>::NT_FWD, smem_slab(K, K), s, d, STAGE_FWD, CS); \
         else                                                                                                     \
-            launch_pdl(k_inv_c<K, CS>, (unsigned)(count * CS), SlabSplit<K, CS>::NT_INV, smem_inv(K, K), s, d,  \
-                       STAGE_INV, CS);                                                                           \
+            launch_pdl(k_inv_c<K, CS>, (unsigned)(count * CS), SlabSplit<K, CS>::NT_INV, smem_inv(K, K), s, d, STAGE_INV, CS);  \
         return true;                                                                                             \
     }
     PME_SPLIT_KS(PME_SPLIT_LAUNCH)
@@ -222,12 +222,12 @@ void launch_stage(const SysDev &d0, int stage, cudaStream_t s) {
             break;
         case STAGE_FWD:
             if (!launch_split_slab(d, true, d.K1, s))
-                launch_pdl(fwd_kernel(d), d.K1, NT_SLAB, smem_slab(d.K2, d.K3), s, d, STAGE_FWD);
+                launch_pdl(fwd_kernel(d), d.K1, slab_threads(d), smem_slab(d.K2, d.K3), s, d, STAGE_FWD);
             break;
         case STAGE_CONV:
             if (d.tc_w) {
                 SysDev dp = d;
-                dp.pdl_late = pdl_when(g_launch_mode, STAGE_CONV);
+                dp.pdl_late = pdl_when(g_launch_mode, STAGE_CONV, d);
                 launch_conv_tc(dp, d.tc_w, s);
             } else {
                 launch_pdl(conv_kernel(d), d.nconv, NT_CONV, smem_conv(d.K1, NT_CONV), s, d, STAGE_CONV);
@@ -235,7 +235,7 @@ void launch_stage(const SysDev &d0, int stage, cudaStream_t s) {
             break;
         case STAGE_INV:
             if (!launch_split_slab(d, false, d.K1, s))
-                launch_pdl(inv_kernel(d), d.K1, NT_SLAB, smem_inv(d.K2, d.K3), s, d, STAGE_INV);
+                launch_pdl(inv_kernel(d), d.K1, slab_threads(d), smem_inv(d.K2, d.K3), s, d, STAGE_INV);
             break;
         default:
             if (d.p == 4) launch_tiles_gather<4>(d, s);
@@ -252,13 +252,13 @@ void launch_stage_items(const SysDev &d0, int stage, int first, int count, cudaS
     if (count < 1) return;
     switch (stage) {
         case STAGE_FWD:
-            launch_pdl(fwd_kernel(d), count, NT_SLAB, smem_slab(d.K2, d.K3), s, d, STAGE_FWD);
+            launch_pdl(fwd_kernel(d), count, slab_threads(d), smem_slab(d.K2, d.K3), s, d, STAGE_FWD);
             break;
         case STAGE_CONV:
             launch_pdl(conv_kernel(d), count, NT_CONV, smem_conv(d.K1, NT_CONV), s, d, STAGE_CONV);
             break;
         case STAGE_INV:
-            launch_pdl(inv_kernel(d), count, NT_SLAB, smem_inv(d.K2, d.K3), s, d, STAGE_INV);
+            launch_pdl(inv_kernel(d), count, slab_threads(d), smem_inv(d.K2, d.K3), s, d, STAGE_INV);
             break;
         default:
             launch_stage(d0, stage, s);

@@ -12,7 +12,17 @@ namespace pme {
 
 constexpr int GB300_SMS = 152;
 constexpr int NT_BIN = 128;    // threads per CTA for binning (BIN_CHUNK atoms per CTA)
-constexpr int NT_SLAB = SLAB_THREADS;  // threads per CTA for the forward / inverse slab FFT stages
+// Threads of the slab CTAs: SLAB_THREADS, or as many more (up to NT_SLAB) as let both passes run in one round of
+// lanes (the plans are chosen to fit SLAB_THREADS where they can; long edges do not). 108^3, whose passes take 704 and
+// 896 lanes: 70.0 -> 61.9 us an evaluation. A kernel's launch bound is its own count: all bounded at 1024, 64^3 ran
+// 27.6 -> 28.9 us.
+constexpr int NT_SLAB = 1024;
+PME_HD int slab_nt(int pr, int pc) {  // lane plans of the rows (K3/2 points) and the columns (K2 points)
+    const int K2 = plan_L(pc) * plan_E(pc), H3 = plan_L(pr) * plan_E(pr) + 1;
+    const int rows = plan_units(pr, K2), cols = plan_units(pc, H3), most = rows > cols ? rows : cols;
+    return most < SLAB_THREADS ? SLAB_THREADS : (most > NT_SLAB ? NT_SLAB : most);
+}
+inline unsigned slab_threads(const SysDev &d) { return (unsigned)slab_nt(d.lp_rows, d.lp_cols); }
 constexpr int NT_TILE = 256;   // threads per CTA for spreading and force interpolation (two per atom), at most,
 constexpr int NT_TILE16 = 512; // with 8^3 / 16^3 tiles
 PME_HD int tile_nt_bound(int T) { return T >= 16 ? NT_TILE16 : NT_TILE; }
@@ -53,15 +63,16 @@ struct Edge {
 };
 
 // Launch mode of the per-stage kernels: 0 plain, 1 programmatic dependent launch triggered at kernel entry,
-// 2 triggered at CTA exit (the influence stage: right after its own wait), 3 triggered right after the
-// kernel's own wait. Process-wide; affects launches recorded afterwards.
+// 2 triggered at CTA exit (see pdl_when for the influence stage), 3 triggered right after the kernel's own wait. Process-wide; affects launches recorded afterwards.
 void set_launch_mode(int mode);
 int launch_mode();
-// The PdlScope argument of a kernel of stage `stage` in launch mode `mode`. In mode 2 the influence stage
-// releases the inverse stage early: the inverse stage's K1 slab CTAs fit beside the influence CTAs and
-// become resident during them (measured 30.6 vs 31.1 us per 64^3 evaluation); released early, the other
-// stages' successors were slower or no faster (their CTAs then land unevenly on the SMs).
-int pdl_when(int mode, int stage);
+// The PdlScope argument of a kernel of stage `stage` of system d in launch mode `mode`. In mode 2 a stage releases
+// its successor at CTA exit, except the influence stage of meshes with K1 <= 64, which releases the inverse stage
+// right after its own wait: those few slab CTAs fit beside the influence CTAs and are resident when they finish
+// (evaluations of single graphs at 64^3 32.4 -> 32.0 us, 48^3 20.6 -> 20.4). More or larger slabs get in the way of the
+// influence CTAs (with / without the early release: 80^3 45.2 / 41.3 us an evaluation, 96^3 52.1 / 45.7, 108^3
+// 80.2 / 70.0, 96 x 90 x 108 81.7 / 75.2). Other stages' successors were slower or no faster when released early.
+int pdl_when(int mode, int stage, const SysDev &d);
 
 // CTAs per slab of the single-system forward and inverse slab stages: 1, or 2 / 4 (a thread-block cluster
 // per slab exchanging its intermediate rows / columns through distributed shared memory; meshes with
