@@ -12,7 +12,7 @@
 // loading the library holds until exit. Every kernel a call may need is loaded by the first call on a device
 // (loading one later could take device memory).
 //
-// 2048 atoms, 32^3, p = 4: 60 us a call. One cooperative kernel with nine grid barriers, its table from
+// 2048 atoms, 32^3, p = 4: 52 us a call. One cooperative kernel with nine grid barriers, its table from
 // a division and two exponentials more per point and its transforms in shared memory took 97 us (88 on the GPU).
 #include <cuda_runtime.h>
 #include <string.h>
@@ -30,7 +30,7 @@ namespace pme {
 constexpr size_t NOALLOC_SCRATCH_BYTES = (size_t)4 << 20;  // 4 MiB per device
 constexpr int NOALLOC_MAX_MESH_POINTS = 32768;             // K1 * K2 * K3 (e.g. 32^3)
 constexpr int64_t NOALLOC_MAX_ATOMS = 16384;
-constexpr int NOALLOC_THREADS = 256;
+constexpr int NOALLOC_THREADS = 128;
 constexpr int NOALLOC_MAX_EDGE = 64;
 
 }  // namespace pme
@@ -43,7 +43,7 @@ namespace pme {
 
 struct NoallocArgs {
     int K1, K2, K3, H3;
-    double recip[9];  // a*_alpha[j] at 3*alpha + j
+    double g[6];      // |m'|^2 = g0 m1^2 + g1 m2^2 + g2 m3^2 + g3 m1 m2 + g4 m1 m3 + g5 m2 m3
     double fac;       // pi^2 / beta^2
     double inv_piv;   // 1 / (pi V)
     float4 *bc;       // influence table (SysDev::bc)
@@ -65,51 +65,47 @@ __host__ __device__ constexpr double spline_knot(int x) {
 __device__ __forceinline__ int dev_signed_freq(int m, int K) { return 2 * m <= K ? m : m - K; }
 
 __device__ __forceinline__ double dev_norm2(const NoallocArgs &A, int mt1, int mt2, int mt3) {
-    const double *r = A.recip;
-    double s = 0.0;
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-        const double v = mt1 * r[j] + mt2 * r[3 + j] + mt3 * r[6 + j];
-        s += v * v;
-    }
-    return s;
+    const double x = mt1, y = mt2, z = mt3;
+    return fma(x, fma(A.g[0], x, fma(A.g[3], y, A.g[4] * z)), fma(y, fma(A.g[1], y, A.g[5] * z), A.g[2] * z * z));
 }
 
 // Clears the charge mesh, counters, partials and control block, and writes the twiddles and the influence table,
-// all in FP64 rounded once. Each block keeps the spline denominators of the three axes in shared memory: with the
-// knots symmetric about P / 2, |sum_k M_P(k + 1) exp(2 pi i m k / K)| = |M_P(P/2) + 2 sum_d M_P(P/2 + d)
-// cos(2 pi m d / K)|. A table point costs one exponential and one division, and as much again on Nyquist planes;
-// the FP64 pipe (1/64 of FP32) bounds this kernel, about 3 us at 32^3.
+// all in FP64 rounded once. Each block keeps B's factors of the three axes in shared memory: with the knots
+// symmetric about P / 2, |sum_k M_P(k + 1) exp(2 pi i m k / K)| = |M_P(P/2) + 2 sum_d M_P(P/2 + d) cos(2 pi m d / K)|.
+// The FP64 pipe (1/64 of FP32: a warp's instruction holds it for 64 cycles) bounds this kernel, so what counts is the
+// number of FP64 instructions in a row of one warp per scheduler: 128 threads a block and a point a thread at 32^3
+// (256 threads left half the blocks without points, 13.9 -> 7.9 us), one exponential and one division a point, and
+// as much again on Nyquist planes; the last block, which has the fewest points, takes the twiddles.
 template <int P>
 __global__ void __launch_bounds__(NOALLOC_THREADS) k_noalloc_setup(NoallocArgs A) {
-    __shared__ double den[3 * NOALLOC_MAX_EDGE];
+    __shared__ double bm[3 * NOALLOC_MAX_EDGE];
     pdl_wait();
     const int tid = threadIdx.x, nth = blockDim.x, gtid = blockIdx.x * nth + tid, gnth = gridDim.x * nth;
     for (int i = gtid; i < A.nzero; i += gnth) A.zero[i] = 0ull;
     const int K1 = A.K1, K2 = A.K2, K3 = A.K3, H3 = A.H3, Nh = K3 / 2;
     constexpr double knots[4] = {spline_knot<P>(P / 2), spline_knot<P>(P / 2 + 1), spline_knot<P>(P / 2 + 2), spline_knot<P>(P / 2 + 3)};
-    for (int i = tid; i < 3 * NOALLOC_MAX_EDGE; i += nth) {
-        const int al = i / NOALLOC_MAX_EDGE, m = i - al * NOALLOC_MAX_EDGE, K = al == 0 ? K1 : (al == 1 ? K2 : K3);
-        if (m < K) {
-            double s = knots[0];
+    for (int i = tid; i < K1 + K2 + H3; i += nth) {
+        const int al = i < K1 ? 0 : (i < K1 + K2 ? 1 : 2), m = i - (al == 0 ? 0 : (al == 1 ? K1 : K1 + K2));
+        const int K = al == 0 ? K1 : (al == 1 ? K2 : K3);
+        double s = knots[0];
 #pragma unroll
-            for (int k = 1; k < P / 2; ++k) s += 2.0 * knots[k] * cospi(2.0 * (double)((m * k) % K) / (double)K);
-            den[i] = s;
-        }
+        for (int k = 1; k < P / 2; ++k) s += 2.0 * knots[k] * cospi((double)(2 * ((m * k) % K)) / (double)K);
+        bm[al * NOALLOC_MAX_EDGE + m] = 1.0 / (s * s);
     }
-    for (int i = gtid; i < K1 + K2 + Nh + Nh + 1; i += gnth) {
-        int k = i, len = K1;
-        if (k >= K1) {
-            k -= K1, len = K2;
-            if (k >= K2) {
-                k -= K2, len = Nh;
-                if (k >= Nh) k -= Nh, len = K3;
+    if (blockIdx.x == gridDim.x - 1)
+        for (int i = tid; i < K1 + K2 + Nh + Nh + 1; i += nth) {
+            int k = i, len = K1;
+            if (k >= K1) {
+                k -= K1, len = K2;
+                if (k >= K2) {
+                    k -= K2, len = Nh;
+                    if (k >= Nh) k -= Nh, len = K3;
+                }
             }
+            double s, c;
+            sincospi(-2.0 * (double)k / (double)len, &s, &c);
+            A.tw[i] = make_float2((float)c, (float)s);
         }
-        double s, c;
-        sincospi(-2.0 * (double)k / (double)len, &s, &c);
-        A.tw[i] = make_float2((float)c, (float)s);
-    }
     __syncthreads();
     // on the half spectrum, [m2][m1][m3]: B(m) (C(m) + C(-m)) / 2 as (hi, lo) floats, then B C f(m) and, off the
     // self-conjugate planes on a Nyquist plane, B C f(m_p), f = 2 (1 / |m'|^2 + pi^2 / beta^2)
@@ -118,21 +114,19 @@ __global__ void __launch_bounds__(NOALLOC_THREADS) k_noalloc_setup(NoallocArgs A
         double v = 0.0, g = 0.0, gp = 0.0;
         if (m1 | m2 | m3) {
             const int mt1 = dev_signed_freq(m1, K1), mt2 = dev_signed_freq(m2, K2);
-            const double d = den[m1] * den[NOALLOC_MAX_EDGE + m2] * den[2 * NOALLOC_MAX_EDGE + m3], D = d * d;
-            const double nm = dev_norm2(A, mt1, mt2, m3);
-            const double inv = 1.0 / (nm * D);  // B / |m'|^2
+            const double B = bm[m1] * bm[NOALLOC_MAX_EDGE + m2] * bm[2 * NOALLOC_MAX_EDGE + m3] * A.inv_piv;
+            const double nm = dev_norm2(A, mt1, mt2, m3), inv = 1.0 / nm;
             v = exp(-A.fac * nm) * inv;
-            const double f = 2.0 * (inv * D + A.fac);
             if (2 * m1 == K1 || 2 * m2 == K2 || 2 * m3 == K3) {
                 // the index of -m keeps the frequency +K/2 on a Nyquist axis
                 const int p1 = 2 * m1 == K1 ? mt1 : -mt1, p2 = 2 * m2 == K2 ? mt2 : -mt2;
-                const double np = dev_norm2(A, p1, p2, 2 * m3 == K3 ? m3 : -m3);
-                v = 0.5 * (v + exp(-A.fac * np) / (np * D));
+                const double np = dev_norm2(A, p1, p2, 2 * m3 == K3 ? m3 : -m3), inp = 1.0 / np;
+                v = 0.5 * (v + exp(-A.fac * np) * inp);
                 const bool self = m3 == 0 || 2 * m3 == K3;
-                if (!self && (2 * m1 == K1 || 2 * m2 == K2)) gp = v * A.inv_piv * 2.0 * (1.0 / np + A.fac);
+                if (!self && (2 * m1 == K1 || 2 * m2 == K2)) gp = v * B * 2.0 * (inp + A.fac);
             }
-            v *= A.inv_piv;
-            g = v * f;
+            v *= B;
+            g = v * 2.0 * (inv + A.fac);
         }
         const float hi = (float)v;
         A.bc[i] = make_float4(hi, (float)(v - (double)hi), (float)g, (float)gp);
@@ -285,7 +279,12 @@ extern "C" pme_status pme_compute_noalloc(const int K[3], int p, double beta, co
     A.K2 = K[1];
     A.K3 = K[2];
     A.H3 = d.H3;
-    memcpy(A.recip, recip, sizeof(recip));
+    for (int al = 0; al < 3; ++al)
+        for (int be = al; be < 3; ++be) {
+            double dot = 0.0;
+            for (int j = 0; j < 3; ++j) dot += recip[3 * al + j] * recip[3 * be + j];
+            A.g[al == be ? al : (al == 0 ? 2 + be : 5)] = al == be ? dot : 2.0 * dot;
+        }
     A.fac = PI_D * PI_D / (beta * beta);
     A.inv_piv = 1.0 / (PI_D * vol);
     A.zero = (unsigned long long *)b;
