@@ -55,9 +55,10 @@ def parse():
 
 TRAFFIC_SOURCES = ["paper_2009_12617_gb300/csrc/common.cuh", "paper_2009_12617_gb300/csrc/fft.cuh",
                    "paper_2009_12617_gb300/csrc/stages.cuh", "paper_2009_12617_gb300/csrc/kernels.h",
-                   "paper_2009_12617_gb300/csrc/kernels.cu", "paper_2009_12617_gb300/csrc/pdl.cuh"]
-STAGE_OF_KERNEL = (("k_bin", "bin"), ("k_spread", "spread"), ("k_fwd", "fft_fwd"), ("k_conv", "influence"),
-                   ("k_inv", "fft_inv"), ("k_gather", "gather"))
+                   "paper_2009_12617_gb300/csrc/kernels.cu", "paper_2009_12617_gb300/csrc/pdl.cuh",
+                   "paper_2009_12617_gb300/csrc/slab_kernels.cuh", "paper_2009_12617_gb300/csrc/conv.cu"]
+STAGE_OF_KERNEL = (("k_bin", "bin"), ("k_spread", "spread"), ("k_slab<Fwd", "fft_fwd"), ("k_conv", "influence"),
+                   ("k_slab<Inv", "fft_inv"), ("k_gather", "gather"))
 
 
 def write_traffic(csv_path: str) -> None:
