@@ -301,7 +301,9 @@ pme_status pme_real_reserve(pme_real *rs, int64_t n);
  * written to forces (accumulate = 0) or added to it (accumulate != 0, e.g. after pme_enqueue on the same
  * stream wrote the reciprocal forces). When ev_dev (DEVICE, 8 doubles) is not NULL it receives (E_real,
  * E_self, virial[6]) when the stream reaches that point. Results are bit-reproducible run to run and do not
- * depend on the order of the atoms except through the summation order of each atom's neighbours. */
+ * depend on the order of the atoms except through the summation order of each atom's neighbours. A non-finite
+ * position or charge, or a position 2^20 cell widths out or more, makes that atom's force and ev_dev NaN (other
+ * forces may be NaN too); the next pme_real_compute on the context returns PME_EINVAL for it. */
 pme_status pme_real_enqueue(pme_real *rs, const float *pos, const float *q, int64_t n, float *forces, int accumulate,
                             double *ev_dev);
 

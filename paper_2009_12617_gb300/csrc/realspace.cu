@@ -98,36 +98,42 @@ __device__ __forceinline__ int image_offset(const RealDev &d, int k, int m0, int
 __device__ __forceinline__ int floordiv(int a, int b) { return a >= 0 ? a / b : -((-a + b - 1) / b); }
 
 // 1: per atom its cell and arrival number, and its fixed-point position: x / u rounded to an integer (exact
-// wherever x's own spacing is at least u), less the whole cells it lies out, both modulo 2^32.
+// wherever x's own spacing is at least u), less the whole cells it lies out, both modulo 2^32. An atom without such
+// a position (a non-finite coordinate, 2^20 cells out) goes to the origin. It and an atom of non-finite charge carry
+// the charge NaN, so that their forces, those around them and the energies show it where nobody asks for the status
+// (pme_real_enqueue).
 __global__ void __launch_bounds__(RS_BIN_THREADS) k_rs_bin(RealDev d) {
     pdl_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < d.n) {
         const float r[3] = {d.pos[3 * (size_t)i], d.pos[3 * (size_t)i + 1], d.pos[3 * (size_t)i + 2]};
         const float qq = d.q[i];
-        int c[3];
-        float fl[3];
-        bool bad = !(isfinite(r[0]) && isfinite(r[1]) && isfinite(r[2]) && isfinite(qq));
+        float s[3];
+        bool lost = !(isfinite(r[0]) && isfinite(r[1]) && isfinite(r[2]));
 #pragma unroll
         for (int al = 0; al < 3; ++al) {
-            const float s = fmaf(r[0], d.rec[3 * al], fmaf(r[1], d.rec[3 * al + 1], r[2] * d.rec[3 * al + 2]));
-            if (!(fabsf(s) < 1048576.0f)) bad = true;  // also catches NaN: absurdly far out
-            fl[al] = bad ? 0.0f : floorf(s);
-            const float f = bad ? 0.0f : s - fl[al];  // exact: s and floor(s) are within one of each other
-            const int ci = (int)(f * (float)d.nc[al]);
-            c[al] = ci < 0 ? 0 : (ci >= d.nc[al] ? d.nc[al] - 1 : ci);
+            s[al] = fmaf(r[0], d.rec[3 * al], fmaf(r[1], d.rec[3 * al + 1], r[2] * d.rec[3 * al + 2]));
+            if (!(fabsf(s[al]) < 1048576.0f)) lost = true;  // also catches NaN: absurdly far out
         }
-        int X[3] = {0, 0, 0};
-        if (bad) {
-            atomicOr(&d.ctl->status, ST_NONFINITE);
-        } else {
+        const bool bad = lost || !isfinite(qq);
+        if (bad) atomicOr(&d.ctl->status, ST_NONFINITE);
+        int c[3] = {0, 0, 0}, X[3] = {0, 0, 0};
+        if (!lost) {
+            int fl[3];
+#pragma unroll
+            for (int al = 0; al < 3; ++al) {
+                const float w = floorf(s[al]), f = s[al] - w;  // exact: s and floor(s) are within one of each other
+                fl[al] = (int)w;
+                const int ci = (int)(f * (float)d.nc[al]);
+                c[al] = ci < 0 ? 0 : (ci >= d.nc[al] ? d.nc[al] - 1 : ci);
+            }
 #pragma unroll
             for (int k = 0; k < 3; ++k)
                 X[k] = wsub((int)(unsigned)(unsigned long long)__double2ll_rn((double)r[k] * d.inv_u),
-                            image_offset(d, k, (int)fl[0], (int)fl[1], (int)fl[2]));
+                            image_offset(d, k, fl[0], fl[1], fl[2]));
         }
         const int cid = (c[0] * d.nc[1] + c[1]) * d.nc[2] + c[2];
-        d.xq[i] = make_int4(X[0], X[1], X[2], __float_as_int(qq));
+        d.xq[i] = make_int4(X[0], X[1], X[2], bad ? 0x7fc00000 : __float_as_int(qq));
         d.cell[i] = make_int2(cid, (int)atomicAdd(d.count + cid, 1u));
     }
 }

@@ -98,6 +98,37 @@ def test_empty_and_invalid(pme, oracle_mod):
     assert ei.value.status == pme.PME_EUNSUPPORTED
 
 
+@pytest.mark.parametrize("what", ["nan_position", "inf_position", "far_position", "nan_charge", "inf_charge"])
+@pytest.mark.parametrize("n", [40, 2048])
+def test_bad_atom_shows_in_asynchronous_results(pme, what, n):
+    """pme_real_enqueue returns no status of the atoms, so an atom without a usable position or charge makes its own
+    force, both energies and the virial NaN; the next synchronous call on the context reports it, and the one after
+    that is clean again. 40 atoms keep far from the cell's origin, where a bad atom must not pass for an ordinary one."""
+    dev = torch.device("cuda:0")
+    box = np.eye(3) * 40.0
+    rng = np.random.default_rng(5)
+    pos = ((15.0 + 10.0 * rng.random((n, 3))) if n == 40 else 40.0 * rng.random((n, 3))).astype(np.float32)
+    q = rng.normal(size=n).astype(np.float32)
+    good = torch.from_numpy(pos).to(dev), torch.from_numpy(q).to(dev)
+    if what.endswith("position"):
+        pos[7, 1] = {"nan": np.nan, "inf": np.inf, "far": 40.0 * 2.0 ** 21}[what[:3]]
+    else:
+        q[7] = np.nan if what == "nan_charge" else np.inf
+    P, Q = torch.from_numpy(pos).to(dev), torch.from_numpy(q).to(dev)
+    F, ev = torch.zeros_like(P), torch.zeros(8, dtype=torch.float64, device=dev)
+    rs = pme.pme_real_create(box, 0.34, 9.0)
+    try:
+        pme.pme_real_enqueue(rs, P, Q, F, ev_dev=ev)
+        assert torch.isnan(ev).all() and torch.isnan(F[7]).all()
+        with pytest.raises(pme.PMEError) as ei:
+            pme.pme_real_compute(rs, P, Q, F)
+        assert ei.value.status == pme.PME_EINVAL
+        er, es, vir = pme.pme_real_compute(rs, *good, F)
+        assert math.isfinite(er) and math.isfinite(es) and np.isfinite(vir).all() and torch.isfinite(F).all()
+    finally:
+        pme.pme_real_destroy(rs)
+
+
 def test_full_ewald_madelung_on_gpu(pme):
     """NaCl rock salt (a = 5.64 A, 2x2x2 conventional cells, 64 ions): GPU SPME reciprocal energy + GPU real
     space + GPU self term = -M N_pairs / (a/2) with the Madelung constant M = 1.747565."""
