@@ -75,6 +75,44 @@ def test_noalloc_matches_pme_compute_twice(name):
         assert rel_virial(V, V_ref) < V_TOL
 
 
+_FIRST_CALLS = """
+import sys
+sys.path.insert(0, {root!r})
+import numpy as np, torch
+from paper_2009_12617_gb300 import pme
+edges = [8, 10, 12, 16, 18, 20, 24, 30, 32, 36, 40, 48, 50, 54, 60, 64]
+pos = torch.rand(50, 3, device="cuda") * 20.0
+q = torch.linspace(-1.0, 1.0, 50, device="cuda")
+F = torch.empty_like(pos)
+def call(K, p):
+    pme.pme_compute_noalloc(K, p, 0.34, np.diag(np.array(K, float)), pos, q, F)
+call((32, 32, 32), 4)
+free = torch.cuda.mem_get_info()[0]
+n = 0
+for K2 in edges:
+    for K3 in edges:
+        for K1 in edges:
+            if K1 * K2 * K3 <= 32768 and (K1 == 8 or K2 == K3 == 8):
+                call((K1, K2, K3), (4, 6, 8)[n % 3])
+                n += 1
+print(n, free - torch.cuda.mem_get_info()[0])
+"""
+
+
+def test_noalloc_later_calls_take_no_device_memory():
+    """In a fresh process, after one call, calls on meshes of every other accepted pair (K2, K3) and of every K1, at all
+    three orders, leave the free device memory as it is: no kernel is left to be loaded."""
+    import os
+    import subprocess
+    import sys
+
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", _FIRST_CALLS.format(root=root)], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr
+    n, taken = (int(x) for x in r.stdout.split())
+    assert n > 150 and taken == 0, r.stdout
+
+
 def test_noalloc_rejects_mismatched_arrays():
     from paper_2009_12617_gb300 import pme
 
