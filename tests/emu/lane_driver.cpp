@@ -1,0 +1,24 @@
+// Lane plans of the register transforms and the launch rules that go by them, compiled for the CPU (tests only).
+#define PME_HOST_EMULATION 1
+#include <stdint.h>
+#include <string.h>
+
+#include "../../paper_2009_12617_gb300/csrc/host_tables.h"
+#include "../../paper_2009_12617_gb300/csrc/kernels.h"
+
+using namespace pme;
+
+extern "C" {
+
+int lane_edges(int *out) {
+    for (int i = 0; i < N_EDGES; ++i) out[i] = mesh_edge(i);
+    return N_EDGES;
+}
+
+// Threads of the slab CTAs of a K2 x K3 slab, for one system or a group of them.
+int lane_slab_threads(int K2, int K3, int group) {
+    const int pr = slab_lane_plan(K3 / 2, K2), pc = slab_lane_plan(K2, K3 / 2 + 1);
+    return group ? slab_group_nt(pr, pc) : slab_nt(pr, pc);
+}
+
+}  // extern "C"

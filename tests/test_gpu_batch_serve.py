@@ -336,3 +336,29 @@ def test_batch_and_server_odd_order(pme, oracle_mod):
     finally:
         for o in syst:
             pme.pme_destroy(o["plan"])
+
+
+@pytest.mark.parametrize("K", [(80, 80, 80), (100, 100, 100), (108, 108, 108), (64, 64, 128), (64, 128, 64), (128, 8, 128)],
+                         ids=lambda K: "x".join(map(str, K)))
+def test_group_slab_threads_keep_the_bits(pme, K):
+    """Groups whose slab CTAs have fewer threads than a single system's (up to 10000 points a slab), and some either
+    side of that line: every system equals its single evaluation bit for bit."""
+    syst = _shaped_systems(pme, [(3000, K, 4), (2500, K, 4)], 600)
+    try:
+        pos, q, ns = packed(syst)
+        F = torch.full_like(pos, float("nan"))
+        ev = torch.zeros((len(syst), 7), dtype=torch.float64, device="cuda:0")
+        b = pme.pme_batch_create([o["plan"] for o in syst], ns)
+        try:
+            pme.pme_batch_set_strategy(b, pme.PME_BATCH_GROUPED)
+            pme.pme_batch_enqueue(b, pos, q, F, ev)
+            pme.pme_batch_sync(b)
+            Fh, evh = F.cpu().numpy(), ev.cpu().numpy()
+            for i, o in enumerate(syst):
+                off = sum(ns[:i])
+                check_same(o, Fh[off:off + ns[i]], evh[i, 0], evh[i, 1:], exact=True)
+        finally:
+            pme.pme_batch_destroy(b)
+    finally:
+        for o in syst:
+            pme.pme_destroy(o["plan"])
