@@ -23,16 +23,17 @@ PME_HD int slab_nt(int pr, int pc) {  // lane plans of the rows (K3/2 points) an
     return most < SLAB_THREADS ? SLAB_THREADS : (most > NT_SLAB ? NT_SLAB : most);
 }
 inline unsigned slab_threads(const SysDev &d) { return (unsigned)slab_nt(d.lp_rows, d.lp_cols); }
-// The same for a group of systems, which has CTAs enough to fill the GPU: SLAB_THREADS for slabs of up to
-// SLAB_GROUP_POINTS points, so that several of them share an SM, slab_nt beyond. us a batch of eight systems of 0.1
-// atoms a point with slab_nt / SLAB_THREADS: 80^3 220 / 211, 80 x 80 x 96 268 / 254, 64 x 64 x 128 233 / 221, 96^3
-// 354 / 339, 100^3 418 / 401, but 108^3 525 / 547 and 128^3 804 / 810.
+// The same for a group of systems with `slabs` slabs in all. Where there are more than one per SM, several CTAs have to
+// share an SM: SLAB_THREADS for slabs of up to SLAB_GROUP_POINTS points. us a batch of eight systems of 0.1 atoms a
+// point with slab_nt / SLAB_THREADS: 80^3 220 / 211, 80 x 80 x 96 268 / 254, 64 x 64 x 128 233 / 221, 96^3 354 / 339,
+// 100^3 418 / 401, but 108^3 525 / 547 and 128^3 804 / 810; of two systems: 80^3 82 / 80, 96^3 111 / 108, but 64 x 128 x 64
+// (128 slabs) 78 / 87.
 constexpr int SLAB_GROUP_POINTS = 10000;
-PME_HD int slab_group_nt(int pr, int pc) {
+PME_HD int slab_group_nt(int pr, int pc, int slabs) {
     const int K2 = plan_L(pc) * plan_E(pc), K3 = 2 * plan_L(pr) * plan_E(pr);
-    return K2 * K3 <= SLAB_GROUP_POINTS ? SLAB_THREADS : slab_nt(pr, pc);
+    return slabs > GB300_SMS && K2 * K3 <= SLAB_GROUP_POINTS ? SLAB_THREADS : slab_nt(pr, pc);
 }
-inline unsigned slab_group_threads(const SysDev &d) { return (unsigned)slab_group_nt(d.lp_rows, d.lp_cols); }
+inline unsigned slab_group_threads(const SysDev &d, int nsys) { return (unsigned)slab_group_nt(d.lp_rows, d.lp_cols, nsys * d.K1); }
 constexpr int NT_TILE = 256;   // threads per CTA for spreading and force interpolation (two per atom), at most,
 constexpr int NT_TILE16 = 512; // with 8^3 / 16^3 tiles
 PME_HD int tile_nt_bound(int T) { return T >= 16 ? NT_TILE16 : NT_TILE; }

@@ -29,9 +29,8 @@ struct SlabPlans {
     static_assert(PR >= 0 && PC >= 0, "every edge has lane plans");
 };
 
-// Launch bounds of the kernels of a pair of plans (-1: any).
+// Launch bound of the kernel of a pair of plans (-1: any).
 constexpr int slab_bound(int pr, int pc) { return pr < 0 ? NT_SLAB : slab_nt(pr, pc); }
-constexpr int slab_group_bound(int pr, int pc) { return pr < 0 ? NT_SLAB : slab_group_nt(pr, pc); }
 
 // Stage is a class with static device functions run<PR, PC>(d, item, smem).
 template <class Stage, int PR, int PC>
@@ -41,7 +40,7 @@ __global__ void __launch_bounds__(slab_bound(PR, PC)) k_slab(SysDev d) {
     Stage::template run<PR, PC>(d, d.item0 + blockIdx.x, smem);
 }
 template <class Stage, int PR, int PC>
-__global__ void __launch_bounds__(slab_group_bound(PR, PC)) k_slab_g(GroupArgs a) {
+__global__ void __launch_bounds__(slab_bound(PR, PC)) k_slab_g(GroupArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ SysDev sd;
     PdlScope pdl(a.late);

@@ -15,10 +15,10 @@ int lane_edges(int *out) {
     return N_EDGES;
 }
 
-// Threads of the slab CTAs of a K2 x K3 slab, for one system or a group of them.
-int lane_slab_threads(int K2, int K3, int group) {
+// Threads of the slab CTAs of K2 x K3 slabs: of a single system (slabs 0), or of a group with that many.
+int lane_slab_threads(int K2, int K3, int slabs) {
     const int pr = slab_lane_plan(K3 / 2, K2), pc = slab_lane_plan(K2, K3 / 2 + 1);
-    return group ? slab_group_nt(pr, pc) : slab_nt(pr, pc);
+    return slabs ? slab_group_nt(pr, pc, slabs) : slab_nt(pr, pc);
 }
 
 }  // extern "C"

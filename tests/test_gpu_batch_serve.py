@@ -338,12 +338,12 @@ def test_batch_and_server_odd_order(pme, oracle_mod):
             pme.pme_destroy(o["plan"])
 
 
-@pytest.mark.parametrize("K", [(80, 80, 80), (100, 100, 100), (108, 108, 108), (64, 64, 128), (64, 128, 64), (128, 8, 128)],
+@pytest.mark.parametrize("K", [(80, 80, 80), (100, 100, 100), (108, 108, 108), (64, 64, 128), (64, 128, 64), (50, 128, 64), (128, 8, 128)],
                          ids=lambda K: "x".join(map(str, K)))
 def test_group_slab_threads_keep_the_bits(pme, K):
-    """Groups whose slab CTAs have fewer threads than a single system's (up to 10000 points a slab), and some either
-    side of that line: every system equals its single evaluation bit for bit."""
-    syst = _shaped_systems(pme, [(3000, K, 4), (2500, K, 4)], 600)
+    """Groups whose slab CTAs have fewer threads than a single system's (up to 10000 points a slab, more slabs than SMs),
+    and some either side of those lines: every system equals its single evaluation bit for bit."""
+    syst = _shaped_systems(pme, [(3000, K, 4), (2500, K, 4), (2000, K, 4)][:3 if K[0] < 100 else 2], 600)
     try:
         pos, q, ns = packed(syst)
         F = torch.full_like(pos, float("nan"))

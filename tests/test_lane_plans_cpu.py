@@ -28,11 +28,13 @@ def edges(lanes):
 
 
 def test_slab_threads_of_groups(lanes, edges):
-    """A group's slabs of up to 10000 points run on 512 threads, so that several CTAs share an SM; larger ones, and
-    every slab of a single system, on as many whole warps as both passes can use in one round (512 to 1024)."""
+    """A group with more slabs than SMs runs slabs of up to 10000 points on 512 threads, so that several CTAs share an
+    SM; larger ones, fewer slabs, and every slab of a single system run on as many whole warps as both passes can use in
+    one round (512 to 1024)."""
     for K2 in edges:
         for K3 in edges:
-            one, group = lanes.lane_slab_threads(K2, K3, 0), lanes.lane_slab_threads(K2, K3, 1)
+            one = lanes.lane_slab_threads(K2, K3, 0)
             assert 512 <= one <= 1024 and one % 32 == 0
-            assert group == (512 if K2 * K3 <= 10000 else one), (K2, K3)
-    assert lanes.lane_slab_threads(80, 80, 0) > 512 and lanes.lane_slab_threads(108, 108, 1) > 512
+            assert lanes.lane_slab_threads(K2, K3, 153) == (512 if K2 * K3 <= 10000 else one), (K2, K3)
+            assert lanes.lane_slab_threads(K2, K3, 152) == one
+    assert lanes.lane_slab_threads(80, 80, 0) > 512 and lanes.lane_slab_threads(108, 108, 1000) > 512
