@@ -75,6 +75,10 @@ constexpr int LANE_PLANS = 37;
             X(17, 16, 5) X(18, 16, 6) X(19, 16, 8) X(20, 32, 4) X(21, 3, 3) X(22, 3, 5) X(23, 3, 6)       \
                 X(24, 5, 5) X(25, 3, 9) X(26, 5, 6) X(27, 6, 6) X(28, 5, 9) X(29, 10, 5) X(30, 6, 9)      \
                     X(31, 10, 6) X(32, 9, 8) X(33, 10, 9) X(34, 10, 10) X(35, 12, 9) X(36, 15, 8)
+// The first LANE_POW2_PLANS plans have a power of two of lanes.
+constexpr int LANE_POW2_PLANS = 21;
+// Plans of a stage body that picks them at run time: among all of them, each a call, or among the first, inlined.
+constexpr int PLAN_ANY = -1, PLAN_POW2 = -2;
 // Threads (lanes) per influence-stage work item on the register path: four warps of 32 / L (rounded down)
 // columns of L lanes each.
 constexpr int CONV_UNITS = 128;

@@ -105,9 +105,9 @@ cudaError_t launch_group_chain(const SysDev *sys_dev, int nsys, const SysDev &pr
                 e = launch_ex(spread_g(d), grid, (unsigned)tile_threads(d, (int64_t)max_nbin * BIN_CHUNK),
                               smem_spread(d.p, d.tlog), s, a);
                 break;
-            case STAGE_FWD: e = launch_ex(fwd_group_kernel(d), grid, slab_nt, smem_slab(d.K2, d.K3), s, a); break;
+            case STAGE_FWD: e = launch_ex(fwd_group_kernel(d, slab_nt), grid, slab_nt, smem_slab(d.K2, d.K3), s, a); break;
             case STAGE_CONV: e = launch_ex(conv_group_kernel(d), grid, NT_CONV, smem_conv(d.K1, NT_CONV), s, a); break;
-            case STAGE_INV: e = launch_ex(inv_group_kernel(d), grid, slab_nt, smem_inv(d.K2, d.K3), s, a); break;
+            case STAGE_INV: e = launch_ex(inv_group_kernel(d, slab_nt), grid, slab_nt, smem_inv(d.K2, d.K3), s, a); break;
             default:
                 e = launch_ex(gather_g(d), grid, (unsigned)tile_threads(d, (int64_t)max_nbin * BIN_CHUNK, true),
                               smem_gather_all(d.p, d.tlog), s, a);

@@ -15,10 +15,11 @@ struct GroupArgs {
 };
 
 using GroupKernel = void (*)(GroupArgs);
-// The grouped slab and influence kernels for a system's plans (fwd.cu, conv.cu, inv.cu).
-GroupKernel fwd_group_kernel(const SysDev &d);
+// The grouped slab kernels for a system's plans and CTAs of that many threads, and the influence kernel (fwd.cu,
+// conv.cu, inv.cu).
+GroupKernel fwd_group_kernel(const SysDev &d, unsigned threads);
 GroupKernel conv_group_kernel(const SysDev &d);
-GroupKernel inv_group_kernel(const SysDev &d);
+GroupKernel inv_group_kernel(const SysDev &d, unsigned threads);
 // and the shared-memory limits of all of them.
 cudaError_t configure_fwd_group_kernels();
 cudaError_t configure_conv_group_kernels();

@@ -29,8 +29,15 @@ struct SlabPlans {
     static_assert(PR >= 0 && PC >= 0, "every edge has lane plans");
 };
 
-// Launch bound of the kernel of a pair of plans (-1: any).
-constexpr int slab_bound(int pr, int pc) { return pr < 0 ? NT_SLAB : slab_nt(pr, pc); }
+// Launch bound of the kernel of a pair of plans.
+constexpr int slab_bound(int pr, int pc) { return pr == PLAN_ANY ? NT_SLAB : (pr == PLAN_POW2 ? SLAB_THREADS : slab_nt(pr, pc)); }
+
+// Of the kernels that pick the plans at run time, the one with the power-of-two plans inlined serves the meshes that it
+// can: the calls of the other cost them about 1 us of an evaluation (48 x 24 x 96 23.3 -> 22.4 us, 128 x 8 x 128
+// 25.4 -> 22.9, 32 x 32 x 64 22.0 -> 20.8, 12^3 18.7 -> 17.3; 16 x 128 x 16 alone gains from them, 21.7 -> 22.2).
+inline bool slab_pow2(const SysDev &d, unsigned threads) {
+    return d.lp_rows < LANE_POW2_PLANS && d.lp_cols < LANE_POW2_PLANS && threads <= (unsigned)SLAB_THREADS;
+}
 
 // Stage is a class with static device functions run<PR, PC>(d, item, smem).
 template <class Stage, int PR, int PC>

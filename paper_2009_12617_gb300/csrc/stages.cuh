@@ -1326,7 +1326,7 @@ __device__ __noinline__ void inv_rows_call(float *phi, int K2, int K3, int k1, i
 
 // Lane slab / influence stages with the plans fixed at compile time (PR, PC, P1 >= 0: only that plan's code
 // is built into the kernel, which keeps it small enough for the instruction caches) or chosen at run time
-// from the system's plans (-1).
+// from the system's plans (PLAN_ANY, PLAN_POW2).
 template <int PR, int PC>
 PME_DEV void stage_fwd_lane(const SysDev &d, int k1, void *smem) {
     const int Nh = d.K3 / 2, zs = d.zs;
@@ -1344,8 +1344,10 @@ PME_DEV void stage_fwd_lane(const SysDev &d, int k1, void *smem) {
     } else {
         switch (d.lp_rows) {
 #define PME_ROWS(c, L, E) \
-    case c:                                                                      \
-        if constexpr (plan_for_rows(c)) fwd_rows_call<L, E>(d.grid, d.tw3h, d.K2, d.K3, k1, zs); \
+    case c:                                                                                                   \
+        if constexpr (plan_for_rows(c) && PR == PLAN_ANY) fwd_rows_call<L, E>(d.grid, d.tw3h, d.K2, d.K3, k1, zs); \
+        else if constexpr (plan_for_rows(c) && c < LANE_POW2_PLANS)                                               \
+            fwd_rows_lane<L, E>(d, k1, SlabDst<1>{{Z}}, zs, 0, d.K2);                                             \
         break;
             PME_LANE_CASES(PME_ROWS)
 #undef PME_ROWS
@@ -1361,8 +1363,10 @@ PME_DEV void stage_fwd_lane(const SysDev &d, int k1, void *smem) {
     } else {
         switch (d.lp_cols) {
 #define PME_COLS(c, L, E) \
-    case c:                                                                                  \
-        if constexpr (plan_for_cols(c)) fwd_cols_call<L, E>(d.spec, d.K2, d.K3, k1, zs); \
+    case c:                                                                                               \
+        if constexpr (plan_for_cols(c) && PC == PLAN_ANY) fwd_cols_call<L, E>(d.spec, d.K2, d.K3, k1, zs); \
+        else if constexpr (plan_for_cols(c) && c < LANE_POW2_PLANS)                                       \
+            fwd_cols_lane<L, E>(d, k1, Z, zs, tw3, tw2, 0, d.H3);                                         \
         break;
             PME_LANE_CASES(PME_COLS)
 #undef PME_COLS
@@ -1390,8 +1394,10 @@ PME_DEV void stage_inv_lane(const SysDev &d, int k1, void *smem) {
     } else {
         switch (d.lp_cols) {
 #define PME_COLS(c, L, E) \
-    case c:                                                                      \
-        if constexpr (plan_for_cols(c)) inv_cols_call<L, E>(d.spec, d.tw2, d.K2, d.K3, k1, ys); \
+    case c:                                                                                                  \
+        if constexpr (plan_for_cols(c) && PC == PLAN_ANY) inv_cols_call<L, E>(d.spec, d.tw2, d.K2, d.K3, k1, ys); \
+        else if constexpr (plan_for_cols(c) && c < LANE_POW2_PLANS)                                              \
+            inv_cols_lane<L, E>(d, k1, SlabDst<1>{{Y}}, ys, 0, d.H3);                                            \
         break;
             PME_LANE_CASES(PME_COLS)
 #undef PME_COLS
@@ -1407,8 +1413,10 @@ PME_DEV void stage_inv_lane(const SysDev &d, int k1, void *smem) {
     } else {
         switch (d.lp_rows) {
 #define PME_ROWS(c, L, E) \
-    case c:                                                                               \
-        if constexpr (plan_for_rows(c)) inv_rows_call<L, E>(d.phi, d.K2, d.K3, k1, ys); \
+    case c:                                                                                              \
+        if constexpr (plan_for_rows(c) && PR == PLAN_ANY) inv_rows_call<L, E>(d.phi, d.K2, d.K3, k1, ys); \
+        else if constexpr (plan_for_rows(c) && c < LANE_POW2_PLANS)                                      \
+            inv_rows_lane<L, E>(d, k1, Y, ys, twh, tw3, 0, d.K2);                                        \
         break;
             PME_LANE_CASES(PME_ROWS)
 #undef PME_ROWS
@@ -1509,9 +1517,10 @@ PME_DEV void stage_conv_lane(const SysDev &d, int item, void *smem) {
 }
 #endif  // PME_LANE_FFT
 
-// Stage entry points: the register path, or the shared-memory path in the CPU emulation. With plans given at compile time (a kernel specialised for one mesh) only their code
-// is built in; such a kernel runs only for systems with exactly those plans.
-template <int PR = -1, int PC = -1>
+// Stage entry points: the register path, or the shared-memory path in the CPU emulation. With plans given at compile
+// time (a kernel specialised for one mesh) only their code is built in; such a kernel runs only for systems with
+// exactly those plans.
+template <int PR = PLAN_ANY, int PC = PLAN_ANY>
 PME_DEV void stage_fwd(const SysDev &d, int k1, void *smem) {
     if (k1 == 0 && PME_TID == 0) d.ctl->novf = 0u;  // spreading (its last reader) has finished
 #if defined(PME_LANE_FFT)
@@ -1530,7 +1539,7 @@ PME_DEV void stage_conv(const SysDev &d, int item, void *smem) {
 #endif
 }
 
-template <int PR = -1, int PC = -1>
+template <int PR = PLAN_ANY, int PC = PLAN_ANY>
 PME_DEV void stage_inv(const SysDev &d, int k1, void *smem) {
 #if defined(PME_LANE_FFT)
     stage_inv_lane<PR, PC>(d, k1, smem);

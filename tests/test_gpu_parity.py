@@ -98,6 +98,10 @@ LANE_EDGES = [(60, 18, 18), (72, 30, 30), (18, 36, 36), (100, 50, 50), (30, 54, 
               (32, 18, 30), (40, 30, 18), (48, 54, 50)]
 
 
+# far from square with power-of-two lanes on both axes: the slab kernels that pick among those plans
+LANE_EDGES += [(48, 24, 96), (128, 8, 128), (16, 10, 12), (8, 8, 8), (12, 80, 20), (40, 128, 16), (20, 16, 64), (24, 96, 40)]
+
+
 @pytest.mark.parametrize("K", LANE_EDGES, ids=["x".join(map(str, K)) for K in LANE_EDGES])
 def test_parity_lane_plans(pmelib, K):
     """The FP64 numpy evaluation (checked against the oracle by the CPU tests) at the parity tolerances."""
