@@ -47,11 +47,10 @@ struct RealCtl {
     double res[8];    // E_real, E_self, virial xx yy zz xy xz yz
 };
 
-struct RealDev {
-    int n;
+// The cells of a box and what goes by them.
+struct RealGrid {
     int nc[3], R[3], ncells;
     int slab, nslab, nrowslabs;  // cells along axis 2 per work-item slab, slabs per row, rows x slabs
-    int max_items;         // launched pair CTAs: n / 32 + one per occupied row slab, at most
     float rec[9];          // a*_alpha[j] at 3 alpha + j (cell assignment)
     int afix[9];           // a_alpha[k] / u at 3 alpha + k, low 32 bits of the nearest integer
     float afrac[9];        // what is left of a_alpha[k] / u, in [-1/2, 1/2]
@@ -59,6 +58,11 @@ struct RealDev {
     float inv_u2;          // 1 / u^2
     float rc2, rc2_slack;        // rcut^2 in units^2, and with the candidate test's relative slack
     float beta04_u, ex_k, c2_u;  // 2 beta u / 5; beta^2 u^2 log2(e); 2 beta u / sqrt(pi)
+};
+
+struct RealDev : RealGrid {
+    int n;
+    int max_items;         // launched pair CTAs: n / 32 + one per occupied row slab, at most
     double beta_d;
     int accumulate;        // forces += (1) or = (0)
     const float *pos, *q;
@@ -693,7 +697,8 @@ struct pme_real {
     cudaStream_t stream = nullptr;
     double box[9] = {0}, recip[9] = {0}, vol = 0.0, beta = 0.0, rcut = 0.0;
     RealDev d;
-    void *cell_mem = nullptr;  // counts, starts, fills, partials, control block (per box)
+    RealGrid fine, coarse;     // the cells for many and for few atoms (real_grid)
+    void *cell_mem = nullptr;  // counts, starts, partials, control block (per box)
     size_t cell_bytes = 0;
     void *atom_mem = nullptr;  // per-atom scratch (grows with n)
     size_t atom_bytes = 0;
@@ -704,32 +709,24 @@ struct pme_real {
 
 static size_t al256r(size_t x) { return (x + 255) & ~(size_t)255; }
 
-// The cells the kernels use: about half a cutoff wide (two per cutoff along axes the cutoff does not span), so
-// that the neighbouring cells -R..R hug the cutoff sphere (around one cell 3.7 instead of 6.4 candidates per
-// pair inside the cutoff), unless that is more than RS_MAX_CELLS of them; then at least a cutoff wide. Rows along
-// axis 2 are cut into slabs of about twenty cells, which bounds a work item's extent. The unit u is the
-// smallest power of two with 2^31 u above every coordinate difference a work item forms: its own extent, R
-// cells and one more.
-static void real_cells(const double box[9], const double recip[9], double rcut, RealDev &d) {
-    for (int sub = 2; sub >= 1; --sub) {
-        long long ncells = 1;
-        for (int al = 0; al < 3; ++al) {
-            const double astar = sqrt(recip[3 * al] * recip[3 * al] + recip[3 * al + 1] * recip[3 * al + 1] +
-                                      recip[3 * al + 2] * recip[3 * al + 2]);
-            const double wfrac = rcut * astar * (1.0 + 1e-6);
-            d.nc[al] = wfrac < 1.0 ? (int)floor(sub / wfrac) : sub;
-            d.R[al] = std::max(1, (int)ceil(wfrac * d.nc[al] - 1e-12));
-            ncells *= d.nc[al];
-        }
-        if (ncells <= RS_MAX_CELLS || sub == 1) {
-            d.ncells = (int)ncells;
-            break;
-        }
+// Cells narrower than the cutoff by the factor sub (sub of them along axes the cutoff spans), in rows along axis 2
+// that are cut into slabs of about `slab` cells, which bounds a work item's extent. The unit u is the smallest power of
+// two with 2^31 u above every coordinate difference a work item forms: its own extent, R cells and one more.
+static double real_cells(const double box[9], const double recip[9], double rcut, int sub, int slab, RealGrid &d) {
+    double ncells = 1.0;
+    for (int al = 0; al < 3; ++al) {
+        const double astar = sqrt(recip[3 * al] * recip[3 * al] + recip[3 * al + 1] * recip[3 * al + 1] +
+                                  recip[3 * al + 2] * recip[3 * al + 2]);
+        const double wfrac = rcut * astar * (1.0 + 1e-6);
+        d.nc[al] = wfrac < 1.0 ? (int)std::min(floor(sub / wfrac), 1e9) : sub;
+        d.R[al] = std::max(1, (int)ceil(wfrac * d.nc[al] - 1e-12));
+        ncells *= d.nc[al];
     }
-    d.nslab = std::max(1, (d.nc[2] + 10) / 20);
+    d.ncells = ncells <= RS_MAX_CELLS ? (int)ncells : 0;
+    d.nslab = std::max(1, (d.nc[2] + slab / 2) / slab);
     d.slab = (d.nc[2] + d.nslab - 1) / d.nslab;
     d.nslab = (d.nc[2] + d.slab - 1) / d.slab;
-    d.nrowslabs = d.nc[0] * d.nc[1] * d.nslab;
+    d.nrowslabs = d.ncells ? d.nc[0] * d.nc[1] * d.nslab : 0;
     double most = 0.0;
     for (int k = 0; k < 3; ++k) {
         double b = 0.0;
@@ -740,34 +737,11 @@ static void real_cells(const double box[9], const double recip[9], double rcut, 
     int e;
     frexp(most * 1.001, &e);  // below 2^e
     d.inv_u = ldexp(1.0, 31 - e);
+    return ncells;
 }
 
-// Checks the cutoff against the box and sets the cell grid and float constants; PME_EUNSUPPORTED when rcut needs more than RS_MAX_R cells per
-// axis or the grid has more than RS_MAX_CELLS cells.
-static pme_status real_geometry(pme_real *rs, const double box[9]) {
-    double recip[9], vol;
-    if (!cell_reciprocal(box, recip, &vol)) return fail(PME_EINVAL, "box is singular");
-    int nc[3], R[3];
-    long long ncells = 1;
-    for (int al = 0; al < 3; ++al) {
-        const double astar = sqrt(recip[3 * al] * recip[3 * al] + recip[3 * al + 1] * recip[3 * al + 1] +
-                                  recip[3 * al + 2] * recip[3 * al + 2]);
-        const double wfrac = rs->rcut * astar * (1.0 + 1e-6);  // cutoff in fractional units, with slack
-        nc[al] = wfrac < 1.0 ? (int)floor(1.0 / wfrac) : 1;
-        if (nc[al] < 1) nc[al] = 1;
-        R[al] = (int)ceil(wfrac * nc[al] - 1e-12);
-        if (R[al] < 1) R[al] = 1;
-        if (R[al] > RS_MAX_R)
-            return fail(PME_EUNSUPPORTED, "rcut %.3g A spans %d cell widths along axis %d (at most %d)", rs->rcut, R[al], al,
-                        RS_MAX_R);
-        ncells *= nc[al];
-    }
-    if (ncells > RS_MAX_CELLS) return fail(PME_EUNSUPPORTED, "%lld cells (at most %d): rcut too small for this box", ncells, RS_MAX_CELLS);
-    memcpy(rs->box, box, sizeof(rs->box));
-    memcpy(rs->recip, recip, sizeof(recip));
-    rs->vol = vol;
-    RealDev &d = rs->d;
-    real_cells(box, recip, rs->rcut, d);
+// The grid's constants that follow from its unit.
+static void real_units(const double box[9], const double recip[9], double beta, double rcut, RealGrid &d) {
     for (int al = 0; al < 3; ++al)
         for (int j = 0; j < 3; ++j) {
             d.rec[3 * al + j] = (float)recip[3 * al + j];
@@ -775,18 +749,60 @@ static pme_status real_geometry(pme_real *rs, const double box[9]) {
             d.afix[3 * al + j] = (int)(unsigned)(unsigned long long)(long long)i;
             d.afrac[3 * al + j] = (float)(v - i);
         }
-    const double u = 1.0 / d.inv_u, rcu = rs->rcut * d.inv_u;
+    const double u = 1.0 / d.inv_u, rcu = rcut * d.inv_u;
     d.inv_u2 = (float)(d.inv_u * d.inv_u);
     d.rc2 = (float)(rcu * rcu);
     d.rc2_slack = (float)(rcu * rcu * (1.0 + 2e-5));
-    d.beta04_u = (float)(0.4 * rs->beta * u);
-    d.ex_k = (float)(rs->beta * rs->beta * u * u * 1.4426950408889634074);
-    d.c2_u = (float)(2.0 * rs->beta * u / 1.7724538509055160273);
+    d.beta04_u = (float)(0.4 * beta * u);
+    d.ex_k = (float)(beta * beta * u * u * 1.4426950408889634074);
+    d.c2_u = (float)(2.0 * beta * u / 1.7724538509055160273);
+}
+
+// The cells for n atoms: about half a cutoff wide, so that the neighbouring cells -R..R hug the cutoff sphere (3.7
+// instead of 6.4 candidates per pair inside the cutoff), where there are no more of them than atoms; at least a cutoff
+// wide otherwise, or where the box has more than RS_MAX_CELLS of the others. With fewer atoms than cells, the scan of
+// the cells and work items of an atom or two are what counts: us with fine / coarse cells, and of one thread per atom
+// over coarse cells, for 65536 atoms, 9 A cutoff, 0.9 atoms in a fine cell 109 / 58, 174; 0.09 549 / 120, 190; 5 A, 0.2
+// 366 / 92, 150; 2048 atoms, 9 A, 0.09 48 / 24, 65. The line would lie at about 4 for uniform systems (2.7 atoms 96 / 74,
+// 6.5 atoms at 12 A 117 / 122), but a droplet's neighbourhoods are full whatever its mean (8 times the mean, 2.7 atoms
+// at 12 A: 219 / 251). The atom count alone decides, so a system's sums depend on nothing else.
+static const RealGrid &real_grid(const pme_real *rs, int64_t n) {
+    return rs->fine.ncells && n >= rs->fine.ncells ? rs->fine : rs->coarse;
+}
+// The kernels' arguments for n atoms, but for the caller's arrays.
+static RealDev real_args(const pme_real *rs, int64_t n) {
+    RealDev d = rs->d;
+    (RealGrid &)d = real_grid(rs, n);
+    d.n = (int)n;
+    return d;
+}
+
+// Checks the cutoff against the box and sets the cell grids; PME_EUNSUPPORTED when rcut needs more than RS_MAX_R cells
+// per axis or the grid of cells at least a cutoff wide has more than RS_MAX_CELLS.
+static pme_status real_geometry(pme_real *rs, const double box[9]) {
+    double recip[9], vol;
+    if (!cell_reciprocal(box, recip, &vol)) return fail(PME_EINVAL, "box is singular");
+    RealGrid fine, coarse;
+    // slabs of ten cutoffs, so that both grids have about the same unit
+    const double nfine = real_cells(box, recip, rs->rcut, 2, 20, fine);
+    const double ncells = real_cells(box, recip, rs->rcut, 1, nfine <= RS_MAX_CELLS ? 10 : 20, coarse);
+    for (int al = 0; al < 3; ++al)
+        if (coarse.R[al] > RS_MAX_R)
+            return fail(PME_EUNSUPPORTED, "rcut %.3g A spans %d cell widths along axis %d (at most %d)", rs->rcut, coarse.R[al],
+                        al, RS_MAX_R);
+    if (ncells > RS_MAX_CELLS) return fail(PME_EUNSUPPORTED, "%.0f cells (at most %d): rcut too small for this box", ncells, RS_MAX_CELLS);
+    memcpy(rs->box, box, sizeof(rs->box));
+    memcpy(rs->recip, recip, sizeof(recip));
+    rs->vol = vol;
+    real_units(box, recip, rs->beta, rs->rcut, fine);
+    real_units(box, recip, rs->beta, rs->rcut, coarse);
+    rs->fine = fine;
+    rs->coarse = coarse;
     return PME_OK;
 }
 
 static pme_status real_alloc_cells(pme_real *rs) {
-    const size_t nc = (size_t)rs->d.ncells;
+    const size_t nc = (size_t)std::max(rs->fine.ncells, rs->coarse.ncells);
     size_t off = 0;
     const size_t o_cnt = off;  off = al256r(off + nc * 4);
     const size_t o_st = off;   off = al256r(off + (nc + 1) * 4);
@@ -985,8 +1001,7 @@ pme_status pme::real_enqueue_on(pme_real *rs, cudaStream_t stream, const float *
     DeviceGuard g(rs->dev);
     pme_status st = real_reserve(rs, n);
     if (st != PME_OK) return st;
-    RealDev d = rs->d;
-    d.n = (int)n;
+    RealDev d = real_args(rs, n);
     d.pos = pos;
     d.q = q;
     d.forces = forces;
@@ -1002,8 +1017,7 @@ pme_status pme::real_enqueue_on(pme_real *rs, cudaStream_t stream, const float *
 // The evaluation into the context's own force array, in two parts: forces (the array is returned; n has been
 // reserved), then energies, filed as one row of a table per call.
 const float *pme::real_enqueue_own(pme_real *rs, cudaStream_t stream, const float *pos, const float *q, int64_t n) {
-    RealDev d = rs->d;
-    d.n = (int)n;
+    RealDev d = real_args(rs, n);
     d.pos = pos;
     d.q = q;
     d.forces = d.fown;
@@ -1011,8 +1025,7 @@ const float *pme::real_enqueue_own(pme_real *rs, cudaStream_t stream, const floa
     return d.fown;
 }
 void pme::real_enqueue_file(pme_real *rs, cudaStream_t stream, int64_t n, unsigned *step, double *file, int stride, int rows) {
-    RealDev d = rs->d;
-    d.n = (int)n;
+    RealDev d = real_args(rs, n);
     d.file_step = step;
     d.file = file;
     d.file_stride = stride;

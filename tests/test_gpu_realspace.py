@@ -262,3 +262,69 @@ def test_pair_kernel_clump_and_collapse(pme, oracle_mod):
     r = oracle_mod.ewald_real(pos2.astype(np.float64), q2.astype(np.float64), 0.34, box, rcut=9.0)
     ref = np.delete(r["forces"], 10, 0)
     assert rms_force(F[keep], ref) < F_RMS_TOL
+
+
+def test_gas_costs_no_more_than_liquid(pme):
+    """65536 atoms at a hundredth of the density have a hundredth of the pairs, and must not be held up by empty cells
+    and work items of an atom or two: at most twice the liquid's time (0.9 of it measured, 4 with cells of half a cutoff
+    for both)."""
+    dev = torch.device("cuda:0")
+    n, us = 65536, []
+    stream = torch.cuda.Stream(dev)
+    for density in (0.1, 0.001):
+        L = (n / density) ** (1.0 / 3.0)
+        pos = np.random.default_rng(8).random((n, 3)) * L
+        P = torch.from_numpy(pos.astype(np.float32)).to(dev)
+        Q = torch.from_numpy(np.where(np.arange(n) % 2, 0.5, -0.5).astype(np.float32)).to(dev)
+        F, ev = torch.empty_like(P), torch.zeros(8, dtype=torch.float64, device=dev)
+        rs = pme.pme_real_create(np.eye(3) * L, 0.34, 9.0, stream=stream)
+        try:
+            torch.cuda.synchronize()
+            best = math.inf
+            with torch.cuda.stream(stream):
+                for _ in range(6):
+                    a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                    a.record(stream)
+                    for _ in range(20):
+                        pme.pme_real_enqueue(rs, P, Q, F, ev_dev=ev)
+                    b.record(stream)
+                    torch.cuda.synchronize()
+                    best = min(best, a.elapsed_time(b) / 20 * 1e3)
+            us.append(best)
+        finally:
+            pme.pme_real_destroy(rs)
+    assert us[1] < 2.0 * us[0], us
+
+
+# atoms, cell edge, edge of the part of it that they fill: around the line between fine and coarse cells (as many atoms
+# as fine cells, 1000 of them here), and inhomogeneous systems on the coarse side of it
+DENSITIES = {"just_fine": (1000, 50.0, None), "just_coarse": (999, 50.0, None), "gas": (2000, 400.0, None),
+             "droplet": (1500, 120.0, 25.0), "two_droplets": (1500, 300.0, 25.0)}
+
+
+@pytest.mark.parametrize("name", sorted(DENSITIES))
+def test_real_space_at_any_density(pme, oracle_mod, name):
+    """Energy, forces and virial against the oracle for few atoms a cell, both sides of the choice of cells; each within
+    1e-6 of the same sums of magnitudes (16 FP32 roundings a pair term). beta rcut = 0.5 keeps pairs at the cutoff in
+    sight. two_droplets: across two opposite corners of the cell, so that neighbours are images of each other."""
+    n, L, size = DENSITIES[name]
+    rng = np.random.default_rng(41)
+    pos = rng.random((n, 3)) * (L if size is None else size) + (0.0 if size is None else 3.0)
+    if name == "two_droplets":
+        pos[::2] = L - pos[::2] - 1.0
+        pos[:, 0] = np.where(rng.random(n) < 0.5, pos[:, 0], pos[:, 0] - L)
+    pos = pos.astype(np.float32)
+    q = rng.normal(size=n).astype(np.float32)
+    beta = 0.05
+    er, es, vir, F = gpu_real(pme, pos, q, np.eye(3) * L, beta, 10.0)
+    p64, q64 = pos.astype(np.float64), q.astype(np.float64)
+    oracle_mod.set_threads(16)
+    try:
+        r = oracle_mod.ewald_real(p64, q64, beta, np.eye(3) * L, rcut=10.0)
+        big = oracle_mod.ewald_real(p64, np.abs(q64), beta, np.eye(3) * L, rcut=10.0)
+    finally:
+        oracle_mod.set_threads(1)
+    assert abs(er - r["energy"]) <= E_REL_TOL * big["energy"]
+    assert np.abs(vir - r["virial"]).max() <= E_REL_TOL * np.abs(big["virial"]).max()
+    assert np.abs(F - r["forces"]).max() <= F_RMS_TOL * np.abs(r["forces"]).max()
+    assert es == pytest.approx(oracle_mod.ewald_self(q64, beta), rel=1e-12)
