@@ -57,11 +57,13 @@ constexpr int BCOUNT_STRIDE = 32;
 // Shared-memory accumulation splits each fixed-point contribution v into hi = rn(v / 2^20) and
 // lo = rn(v - hi 2^20) in [-2^19, 2^19], summed in two int32 arrays with native 32-bit atomics. A B-spline
 // weight of order >= 4 is at most 2/3, so with |q| <= Q_TILE_MAX every |v| <= 2 (2/3)^3 2^40 < 2^39, |hi|
-// <= 2^19; with at most 1024 atoms per tile neither sum reaches 2^30. Atoms with larger charges take the
-// 64-bit global path instead. Bucket capacity per tile: at most CAP_MAX (8^3 tiles) or CAP_MAX16 (16^3).
+// <= 2^19; with at most 1024 atoms at a time neither sum reaches 2^30. Atoms with larger charges take the
+// 64-bit global path instead. A tile spreads its bucket CAP_MAX (8^3 tiles) or CAP_MAX16 (16^3) atoms at a time;
+// buckets of 8^3 tiles hold no more than that, those of 16^3 tiles up to BUCKET_MAX16.
 constexpr float Q_TILE_MAX = 2.0f;
 constexpr int CAP_MAX = 512;
 constexpr int CAP_MAX16 = 1024;
+constexpr int BUCKET_MAX16 = 8192;
 constexpr int cap_max_for(int tlog) { return tlog >= 4 ? CAP_MAX16 : CAP_MAX; }
 // Columns m3 per influence-stage work item (shared-memory transform path).
 constexpr int CONV_COLS = 8;

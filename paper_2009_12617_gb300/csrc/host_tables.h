@@ -114,17 +114,28 @@ inline int choose_k1_pieces(const SysDev &d, int sms) {
 
 // Tile edge for n atoms at order p on a GPU with `sms` SMs. 16^3 tiles halve the halo each tile adds to the global
 // mesh (a region of (16 + p - 1)^3 points per 4096 instead of (8 + p - 1)^3 per 512) and there are 8 times fewer of
-// them, so they pay as soon as there is about one per SM, at any density measured (from 48 atoms a tile; below 32,
-// 8^3 is kept). us per evaluation with 8^3 / 16^3 tiles, 152 SMs: p = 6 at 80 x 80 x 96 (150 tiles, 60000 atoms)
+// them, so they pay as soon as there is about one per SM, from 48 atoms a tile (below 32, 8^3 is kept). us per evaluation
+// with 8^3 / 16^3 tiles, 152 SMs: p = 6 at 80 x 80 x 96 (150 tiles, 60000 atoms)
 // 63 / 56, 90 x 96 x 100 (252 tiles) with 12000, 50001 and 80001 atoms 62 / 57, 69 / 58, 73 / 65, 128^3 with 25000 and
 // 262144 atoms 109 / 84, 147 / 126; p = 8 at 80 x 80 x 96 90 / 73; but 80^3 (125 tiles, 120000 atoms) 67 / 79. At p = 4
 // the halo is thin and the 8^3 spreading kernel free of bank conflicts, so that it takes a few more tiles: 72 x 80 x 96
-// (150 tiles, 90000 atoms) 48 / 52, 72 x 80 x 100 (175 tiles) 45.9 / 44.9, 128^3 98 / 90. Results do not depend on the edge.
+// (150 tiles, 90000 atoms) 48 / 52, 72 x 80 x 100 (175 tiles) 45.9 / 44.9, 128^3 98 / 90.
+//
+// A 16^3 tile takes CAP_MAX16 atoms at a time, so with more in a tile the edges come closer: 16^3 stays ahead at p = 6
+// and 8 (90 x 96 x 100 with 252000 and 504000 atoms, p = 8: 178 / 148, 273 / 249), up to about 1150 atoms in a full tile at
+// p = 4 and 5 (p = 4, 226800 and 252000 atoms: 63 / 62, 65 / 67), half as many at p = 4 where tiles are few
+// (72 x 80 x 100, 122500 atoms: 46.3 / 47.8), and again once the buckets of 8^3 tiles run over (90 x 96 x 100, 882000
+// atoms, p = 4: 218 / 131). Results do not depend on the edge.
 inline int choose_tile_log(int64_t n, const int K[3], int sms, int p = 4) {
     const int64_t t16 = (int64_t)((K[0] + 15) / 16) * ((K[1] + 15) / 16) * ((K[2] + 15) / 16);
     const int64_t want = p == 4 ? sms + sms / 8 : sms - sms / 16;
-    if (sms > 0 && t16 >= want && n >= 32 * t16) return TILE_MAX_LOG;
-    return TILE_MIN_LOG;
+    if (sms <= 0 || t16 < want || n < 32 * t16) return TILE_MIN_LOG;
+    if (p <= 5) {
+        const double full = 4096.0 * (double)n / ((double)K[0] * K[1] * K[2]);  // atoms in a tile of all its points
+        const double most = p == 4 && t16 < sms + sms / 3 ? CAP_MAX16 / 2 : CAP_MAX16 * 9 / 8;
+        if (full > most && full < 7 * CAP_MAX) return TILE_MIN_LOG;
+    }
+    return TILE_MAX_LOG;
 }
 
 // Transform paths: the register path (lane plans), or the shared-memory Stockham path for the CPU emulation of the
@@ -311,16 +322,18 @@ inline bool make_slab_layout(const SysDev &d, int P, SlabLayout &L) {
     return true;
 }
 
-// Bucket capacity per tile for n atoms in tiles of edge 2^tlog: twice the mean occupancy plus a margin, a
-// multiple of 32, at most cap_max_for(tlog). Atoms beyond it go to the overflow list (handled by
-// global-memory paths), so this only tunes speed.
-inline int bucket_capacity(int64_t n, int ntiles, int tlog) {
-    const int cmax = cap_max_for(tlog);
-    const double mean = (double)n / (double)ntiles;
-    const double want = 2.0 * mean + 32.0;
-    int cap = want > (double)cmax ? cmax : (int)want;
+// Bucket capacity per tile for n atoms: with 8^3 tiles twice the mean occupancy plus 32, a multiple of 32, at most
+// CAP_MAX; with 16^3 tiles what the eight 8^3 tiles in one would have, at most BUCKET_MAX16. Atoms beyond it go to the
+// overflow list, whose few CTAs are many times slower, so this only tunes speed.
+inline int bucket_capacity(int64_t n, const SysDev &d) {
+    const bool big = d.tlog >= TILE_MAX_LOG;
+    const int tiles = big ? ((d.K1 + 7) / 8) * ((d.K2 + 7) / 8) * ((d.K3 + 7) / 8) : d.ntiles;
+    const int most = big ? BUCKET_MAX16 / 8 : CAP_MAX;
+    const double want = 2.0 * (double)n / (double)tiles + 32.0;
+    int cap = want > (double)most ? most : (int)want;
     cap = (cap + 31) / 32 * 32;
-    return cap < 32 ? 32 : (cap > cmax ? cmax : cap);
+    cap = cap < 32 ? 32 : (cap > most ? most : cap);
+    return big ? 8 * cap : cap;
 }
 
 // Bytes of the padded tile-counter array and of the influence-stage partials.

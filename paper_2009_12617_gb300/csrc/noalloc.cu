@@ -234,7 +234,7 @@ extern "C" pme_status pme_compute_noalloc(const int K[3], int p, double beta, co
     const size_t K1 = K[0], K2 = K[1], K3 = K[2], H3 = d.H3, Nh = K3 / 2;
     const size_t par_bytes = (K2 * (size_t)d.nchunk3 + K1) * 8 * sizeof(float2);
     const int64_t ncap = n > 0 ? n : 1;
-    const int cap = bucket_capacity(ncap, d.ntiles, d.tlog);
+    const int cap = bucket_capacity(ncap, d);
     size_t off = 0;
     const size_t o_ctl = off;  off = al256(off + sizeof(Ctl));
     const size_t o_cnt = off;  off = al256(off + bcount_bytes(d.ntiles));

@@ -158,7 +158,7 @@ pme_status plan_reserve(pme_plan *pl, int64_t n) {
     // between evaluations, so the tiling may change here; results do not depend on it)
     set_tiling(d, pl->tile_log_set ? pl->tile_log_set : choose_tile_log(ncap, pl->K, pl->sms, pl->p));
     set_tiling(d, d.tlog, choose_k1_pieces(d, pl->sms));
-    const int cap = bucket_capacity(ncap, d.ntiles, d.tlog);
+    const int cap = bucket_capacity(ncap, d);
     const size_t nb = (size_t)d.ntiles * cap;
     size_t off = 0;
     const size_t o_bka = off; off = align256(off + nb * 16);

@@ -508,157 +508,167 @@ PME_DEV void stage_spread(const SysDev &d, int item, void *smem, bool cleared = 
     int2 *B = d.bkb + (size_t)item * d.cap;
     // this thread's first record in flight with the count, for the threads below the mean occupancy (the
     // bucket capacity is twice it plus a margin), so that few loads land on empty slots
-    const bool pf = tid < (d.cap >> 1);
+    bool pf = tid < (d.cap >> 1);
     float4 ra0 = make_float4(0.f, 0.f, 0.f, 0.f);
     int2 rb0 = make_int2(0, 0);
     if (pf) {
         ra0 = ldcg(A + tid);
         rb0 = ldcg(B + tid);
     }
-    const int cnt = imin((int)ldcg(&d.bcount[(size_t)item * BCOUNT_STRIDE]), d.cap);
+    const int total = imin((int)ldcg(&d.bcount[(size_t)item * BCOUNT_STRIDE]), d.cap);
     if (!cleared) spread_clear<P, T>(smem);
     PME_SYNC();
-    if constexpr (SpreadLayout<P, T>::WARP) {
-        // one thread per atom: its weights and the region index of its highest support point
-        for (int a = tid; a < cnt; a += nth) {
-            const bool first = pf && a == tid;
-            const float4 ra = first ? ra0 : ldcg(A + a);
-            const int2 rb = first ? rb0 : ldcg(B + a);
-            float th1[P], th2[P], th3[P];
-            bspline_w<P>(ra.x, th1);
-            bspline_w<P>(ra.y, th2);
-            bspline_w<P>(ra.z, th3);
-            const float qs = ra.w * FIX_SCALE;  // exact: a power of two
-            sm.u_s[a] = make_float4(qs * th1[0], qs * th1[2], qs * th1[1], qs * th1[3]);
-            sm.t2_s[a] = make_float4(th2[0], th2[1], th2[2], th2[3]);
-            sm.t3_s[a] = make_float4(th3[0], th3[1], th3[2], th3[3]);
-            sm.ix_s[a] = ((rb.x & 1023) - o1 + H) * PL + (((rb.x >> 10) & 1023) - o2 + H) * RS +
-                         (((rb.x >> 20) & 1023) - o3 + H);
-        }
-        PME_SYNC();
-        // one warp per atom, its 64 points over the 32 lanes (two each, in distinct banks); each warp takes
-        // the atoms w, w + nw, ... two at a time, both atoms' weights loaded before either is added
-#if defined(PME_HOST_EMULATION)
-        for (int a = 0; a < cnt; ++a)
-            for (int lane = 0; lane < 32; ++lane) {
-                const Lanes4<P, T> ln(sm, lane);
-                ln.add(ln.load(a));
-            }
-#else
-        const int nw = nth >> 5;
-        const Lanes4<P, T> ln(sm, tid & 31);
-        int a = tid >> 5;
-        for (; a + nw < cnt; a += 2 * nw) {
-            const Lane4 w0 = ln.load(a), w1 = ln.load(a + nw);
-            ln.add(w0);
-            ln.add(w1);
-        }
-        if (a < cnt) ln.add(ln.load(a));
-#endif
-    } else {
-        // Dealt order: residue r = (base mod 16) of the atom's highest support point in the padded region;
-        // round k takes the k-th atom of every residue in turn, so 16 consecutive atoms (one warp) mostly have
-        // distinct residues and their shared-memory atomics do not share banks. Results do not depend on the
-        // order (integer sums).
-        for (int a = tid; a < cnt; a += nth) {
-            const bool first = pf && a == tid;
-            const float4 ra = first ? ra0 : ldcg(A + a);
-            const int2 rb = first ? rb0 : ldcg(B + a);
-            ra_s[a] = ra;
-            rb_s[a] = rb;
-            const int l1 = (rb.x & 1023) - o1 + H, l2 = ((rb.x >> 10) & 1023) - o2 + H,
-                      l3 = ((rb.x >> 20) & 1023) - o3 + H;
-            const int res = (l1 * PL + l2 * R + l3) & 15;
-            key_s[a] = ((int)atomic_add_u32(bins + res, 1u) << 4) | res;
-        }
-        PME_SYNC();
-        {
-            unsigned nb[16];
-#pragma unroll
-            for (int b = 0; b < 16; ++b) nb[b] = bins[b];
+    for (int done = 0;; done += SpreadLayout<P, T>::CAP) {  // CAP atoms at a time
+        const int cnt = T >= 16 ? imin(total - done, SpreadLayout<P, T>::CAP) : total;
+        if constexpr (SpreadLayout<P, T>::WARP) {
+            // one thread per atom: its weights and the region index of its highest support point
             for (int a = tid; a < cnt; a += nth) {
-                const int key = key_s[a], res = key & 15;
-                const unsigned rk = (unsigned)(key >> 4);
-                unsigned pos = 0;
-#pragma unroll
-                for (int b = 0; b < 16; ++b) pos += (nb[b] < rk ? nb[b] : rk) + ((b < res && nb[b] > rk) ? 1u : 0u);
-                inv_s[pos] = a;
+                const bool first = pf && a == tid;
+                const float4 ra = first ? ra0 : ldcg(A + a);
+                const int2 rb = first ? rb0 : ldcg(B + a);
+                float th1[P], th2[P], th3[P];
+                bspline_w<P>(ra.x, th1);
+                bspline_w<P>(ra.y, th2);
+                bspline_w<P>(ra.z, th3);
+                const float qs = ra.w * FIX_SCALE;  // exact: a power of two
+                sm.u_s[a] = make_float4(qs * th1[0], qs * th1[2], qs * th1[1], qs * th1[3]);
+                sm.t2_s[a] = make_float4(th2[0], th2[1], th2[2], th2[3]);
+                sm.t3_s[a] = make_float4(th3[0], th3[1], th3[2], th3[3]);
+                sm.ix_s[a] = ((rb.x & 1023) - o1 + H) * PL + (((rb.x >> 10) & 1023) - o2 + H) * RS +
+                             (((rb.x >> 20) & 1023) - o3 + H);
             }
-        }
-        PME_SYNC();
-        if (dealt_buckets(P, SpreadLayout<P, T>::TLOG) && cnt >= DEALT_MIN) {
-            for (int pos = tid; pos < cnt; pos += nth) {
-                A[pos] = ra_s[inv_s[pos]];
-                B[pos] = rb_s[inv_s[pos]];
+            PME_SYNC();
+            // one warp per atom, its 64 points over the 32 lanes (two each, in distinct banks); each warp takes
+            // the atoms w, w + nw, ... two at a time, both atoms' weights loaded before either is added
+#if defined(PME_HOST_EMULATION)
+            for (int a = 0; a < cnt; ++a)
+                for (int lane = 0; lane < 32; ++lane) {
+                    const Lanes4<P, T> ln(sm, lane);
+                    ln.add(ln.load(a));
+                }
+#else
+            const int nw = nth >> 5;
+            const Lanes4<P, T> ln(sm, tid & 31);
+            int a = tid >> 5;
+            for (; a + nw < cnt; a += 2 * nw) {
+                const Lane4 w0 = ln.load(a), w1 = ln.load(a + nw);
+                ln.add(w0);
+                ln.add(w1);
             }
-        }
-        // two threads per atom: half 0 takes the planes j1 in [0, H0), half 1 [H0, P)
-        constexpr int H0 = half_planes(P);
-        for (int a2 = tid; a2 < 2 * cnt; a2 += nth) {
-            const int a = inv_s[a2 >> 1], half = a2 & 1;
-            const float4 ra = ra_s[a];
-            const int2 rb = rb_s[a];
-            float th1[P], th2[P], th3[P];
-            bspline_w<P>(ra.x, th1);
-            bspline_w<P>(ra.y, th2);
-            bspline_w<P>(ra.z, th3);
-            // local index of the atom's highest support point; its points are l - j, j < P
-            const int l1 = (rb.x & 1023) - o1 + H;
-            const int l2 = ((rb.x >> 10) & 1023) - o2 + H;
-            const int l3 = ((rb.x >> 20) & 1023) - o3 + H;
+            if (a < cnt) ln.add(ln.load(a));
+#endif
+        } else {
+            // Dealt order: residue r = (base mod 16) of the atom's highest support point in the padded region;
+            // round k takes the k-th atom of every residue in turn, so 16 consecutive atoms (one warp) mostly have
+            // distinct residues and their shared-memory atomics do not share banks. Results do not depend on the
+            // order (integer sums).
+            for (int a = tid; a < cnt; a += nth) {
+                const bool first = pf && a == tid;
+                const float4 ra = first ? ra0 : ldcg(A + a);
+                const int2 rb = first ? rb0 : ldcg(B + a);
+                ra_s[a] = ra;
+                rb_s[a] = rb;
+                const int l1 = (rb.x & 1023) - o1 + H, l2 = ((rb.x >> 10) & 1023) - o2 + H,
+                          l3 = ((rb.x >> 20) & 1023) - o3 + H;
+                const int res = (l1 * PL + l2 * R + l3) & 15;
+                key_s[a] = ((int)atomic_add_u32(bins + res, 1u) << 4) | res;
+            }
+            PME_SYNC();
+            {
+                unsigned nb[16];
 #pragma unroll
-            for (int jj = 0; jj < H0; ++jj) {
-                if (half && jj >= P - H0) break;  // odd P: half 1 has one plane fewer
-                const int j1 = half * H0 + jj;
-                const float t1 = half ? th1[H0 + jj < P ? H0 + jj : P - 1] : th1[jj];
+                for (int b = 0; b < 16; ++b) nb[b] = bins[b];
+                for (int a = tid; a < cnt; a += nth) {
+                    const int key = key_s[a], res = key & 15;
+                    const unsigned rk = (unsigned)(key >> 4);
+                    unsigned pos = 0;
 #pragma unroll
-                for (int j2 = 0; j2 < P; ++j2) {
-                    // scaled row factor: rn(c 2^40 th3) = rn(c th3) 2^40 (a power of two; |v| < 2^62, and values
-                    // small enough for the scaling to matter round to 0 either way), one multiply per point
-                    const float c = ra.w * t1 * th2[j2] * FIX_SCALE;
-                    const int row = (l1 - j1) * PL + (l2 - j2) * R + l3;
+                    for (int b = 0; b < 16; ++b) pos += (nb[b] < rk ? nb[b] : rk) + ((b < res && nb[b] > rk) ? 1u : 0u);
+                    inv_s[pos] = a;
+                }
+            }
+            PME_SYNC();
+            if (dealt_buckets(P, SpreadLayout<P, T>::TLOG) && cnt >= DEALT_MIN) {
+                for (int pos = tid; pos < cnt; pos += nth) {
+                    A[pos] = ra_s[inv_s[pos]];
+                    B[pos] = rb_s[inv_s[pos]];
+                }
+            }
+            // two threads per atom: half 0 takes the planes j1 in [0, H0), half 1 [H0, P)
+            constexpr int H0 = half_planes(P);
+            for (int a2 = tid; a2 < 2 * cnt; a2 += nth) {
+                const int a = inv_s[a2 >> 1], half = a2 & 1;
+                const float4 ra = ra_s[a];
+                const int2 rb = rb_s[a];
+                float th1[P], th2[P], th3[P];
+                bspline_w<P>(ra.x, th1);
+                bspline_w<P>(ra.y, th2);
+                bspline_w<P>(ra.z, th3);
+                // local index of the atom's highest support point; its points are l - j, j < P
+                const int l1 = (rb.x & 1023) - o1 + H;
+                const int l2 = ((rb.x >> 10) & 1023) - o2 + H;
+                const int l3 = ((rb.x >> 20) & 1023) - o3 + H;
 #pragma unroll
-                    for (int j3 = 0; j3 + 1 < P; j3 += 2) {  // two points per paired instruction
-                        int h0, l0, h1, l1;
-                        fix_split2(f2_mul(f2_all(c), f2(th3[j3], th3[j3 + 1])), h0, l0, h1, l1);
-                        shared_add(hi, row - j3, h0);
-                        shared_add(lo, row - j3, l0);
-                        shared_add(hi, row - j3 - 1, h1);
-                        shared_add(lo, row - j3 - 1, l1);
-                    }
-                    if (P & 1) {
-                        int h, l;
-                        fix_split(c * th3[P - 1], h, l);
-                        shared_add(hi, row - P + 1, h);
-                        shared_add(lo, row - P + 1, l);
+                for (int jj = 0; jj < H0; ++jj) {
+                    if (half && jj >= P - H0) break;  // odd P: half 1 has one plane fewer
+                    const int j1 = half * H0 + jj;
+                    const float t1 = half ? th1[H0 + jj < P ? H0 + jj : P - 1] : th1[jj];
+#pragma unroll
+                    for (int j2 = 0; j2 < P; ++j2) {
+                        // scaled row factor: rn(c 2^40 th3) = rn(c th3) 2^40 (a power of two; |v| < 2^62, and values
+                        // small enough for the scaling to matter round to 0 either way), one multiply per point
+                        const float c = ra.w * t1 * th2[j2] * FIX_SCALE;
+                        const int row = (l1 - j1) * PL + (l2 - j2) * R + l3;
+#pragma unroll
+                        for (int j3 = 0; j3 + 1 < P; j3 += 2) {  // two points per paired instruction
+                            int h0, l0, h1, l1;
+                            fix_split2(f2_mul(f2_all(c), f2(th3[j3], th3[j3 + 1])), h0, l0, h1, l1);
+                            shared_add(hi, row - j3, h0);
+                            shared_add(lo, row - j3, l0);
+                            shared_add(hi, row - j3 - 1, h1);
+                            shared_add(lo, row - j3 - 1, l1);
+                        }
+                        if (P & 1) {
+                            int h, l;
+                            fix_split(c * th3[P - 1], h, l);
+                            shared_add(hi, row - P + 1, h);
+                            shared_add(lo, row - P + 1, l);
+                        }
                     }
                 }
             }
         }
-    }
-    PME_SYNC();
-    // flush: thread t < ng R^2 takes the column (i2, i3) = (c / R, c mod R), c = t mod R^2, and adds its
-    // points of the planes i1 = t / R^2, t / R^2 + ng, ... below R1 (the tile's k1 width plus the halo):
-    // the column's mesh address is computed once, each plane costs one add and one wrap
-    constexpr int RR = R * R;
-    const int R1 = tile_width1(d, o1) + H;
-    const int ng = nth >= RR ? nth / RR : 1, g = nth >= RR ? tid / RR : 0;
-    const size_t plane = (size_t)d.K2 * d.K3;
-    if (g < ng) {
-        for (int c = nth >= RR ? tid - g * RR : tid; c < RR; c += nth >= RR ? RR : nth) {
-            const int i2 = c / R, i3 = c - i2 * R;
-            unsigned long long *col = d.grid + (size_t)wrapk(o2 - H + i2, d.K2) * d.K3 + wrapk(o3 - H + i3, d.K3);
-            const int *hc = hi + i2 * RS + i3, *lc = lo + i2 * RS + i3;
-            int k1 = wrapk(o1 - H + g, d.K1);
+        PME_SYNC();
+        // flush: thread t < ng R^2 takes the column (i2, i3) = (c / R, c mod R), c = t mod R^2, and adds its
+        // points of the planes i1 = t / R^2, t / R^2 + ng, ... below R1 (the tile's k1 width plus the halo):
+        // the column's mesh address is computed once, each plane costs one add and one wrap
+        constexpr int RR = R * R;
+        const int R1 = tile_width1(d, o1) + H;
+        const int ng = nth >= RR ? nth / RR : 1, g = nth >= RR ? tid / RR : 0;
+        const size_t plane = (size_t)d.K2 * d.K3;
+        if (g < ng) {
+            for (int c = nth >= RR ? tid - g * RR : tid; c < RR; c += nth >= RR ? RR : nth) {
+                const int i2 = c / R, i3 = c - i2 * R;
+                unsigned long long *col = d.grid + (size_t)wrapk(o2 - H + i2, d.K2) * d.K3 + wrapk(o3 - H + i3, d.K3);
+                const int *hc = hi + i2 * RS + i3, *lc = lo + i2 * RS + i3;
+                int k1 = wrapk(o1 - H + g, d.K1);
 #pragma unroll 4
-            for (int i1 = g; i1 < R1; i1 += ng) {
-                const int h = hc[i1 * PL], l = lc[i1 * PL];
-                // k1 outside [k1_lo, k1_hi): another rank's planes (slab decomposition)
-                if ((h | l) != 0 && k1 >= d.k1_lo && k1 < d.k1_hi) red_add_u64(col + k1 * plane, fix_join(h, l));
-                k1 += ng;
-                if (k1 >= d.K1) k1 -= d.K1;
+                for (int i1 = g; i1 < R1; i1 += ng) {
+                    const int h = hc[i1 * PL], l = lc[i1 * PL];
+                    // k1 outside [k1_lo, k1_hi): another rank's planes (slab decomposition)
+                    if ((h | l) != 0 && k1 >= d.k1_lo && k1 < d.k1_hi) red_add_u64(col + k1 * plane, fix_join(h, l));
+                    k1 += ng;
+                    if (k1 >= d.K1) k1 -= d.K1;
+                }
             }
         }
+        if (T < 16 || done + cnt >= total) return;
+        A += cnt;
+        B += cnt;
+        pf = false;
+        PME_SYNC();
+        spread_clear<P, T>(smem);
+        PME_SYNC();
     }
 }
 

@@ -64,11 +64,14 @@ def main(lib_path):
     run(np.zeros((0, 3)), np.zeros(0), (32, 32, 32), 4, np.diag([20.0] * 3), 0, 0)
     pos = np.full((300, 3), 5.0) + rng.random((300, 3)) * 0.1
     run(pos, rng.normal(size=300), (32, 32, 32), 4, np.diag([20.0] * 3), 0, 0)
+    # 16^3 tiles with more atoms than they take at a time
+    for p in (4, 5, 6, 8):
+        run(rng.random((2500, 3)) * 16.0, rng.normal(size=2500), (16, 16, 16), p, np.diag([16.0] * 3), 0, 4)
     # triclinic cell
     tri = np.array([[20.0, 0, 0], [4.0, 22.0, 0], [-3.0, 5.0, 24.0]])
     pos = rng.random((250, 3)) @ tri
     run(pos, rng.normal(size=250), (24, 30, 32), 6, tri, 0, 0)
-    print(f"asan sweep ok: {cases + 3} cases")
+    print(f"asan sweep ok: {cases + 7} cases")
 
 
 if __name__ == "__main__":

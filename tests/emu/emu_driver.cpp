@@ -88,7 +88,7 @@ static int emu_setup(EmuState &s, int64_t n, const int K[3], int p, double beta,
     s.bcount.assign(bcount_bytes(d.ntiles) / sizeof(unsigned), 0u);
     s.qslot.assign(QABS_BYTES / sizeof(unsigned long long), 0ull);
     s.partials.assign(partials_bytes(d) / sizeof(double), 0.0);
-    const int cap = cap_override > 0 ? cap_override : bucket_capacity(n > 0 ? n : 1, d.ntiles, d.tlog);
+    const int cap = cap_override > 0 ? cap_override : bucket_capacity(n > 0 ? n : 1, d);
     s.bka.resize((size_t)d.ntiles * cap);
     s.bkb.resize((size_t)d.ntiles * cap);
     s.ova.resize(n > 0 ? n : 1);

@@ -82,6 +82,23 @@ def test_emulated_results_do_not_depend_on_tiling(emu):
     assert np.array_equal(F8, F16) and np.array_equal(ev8, ev16)
 
 
+@pytest.mark.parametrize("p", [4, 5, 6, 8])
+@pytest.mark.parametrize("n", [1024, 1025, 2048, 2500])
+def test_emulated_crowded_tile(emu, n, p):
+    """A 16^3 tile with more atoms than it takes at a time (1024): the mesh, forces and energies of 8^3 tiles and of the
+    overflow path bit for bit."""
+    rng = np.random.default_rng(n + p)
+    pos = (rng.random((n, 3)) * 16.0).astype(np.float32)
+    q = rng.normal(size=n).astype(np.float32)
+    box = np.diag([16.0] * 3)
+    ref = emu_spme(emu, pos, q, (16, 16, 16), p, 0.34, box, tile_log=3)
+    for cap in (0, 1024):  # all in the bucket; the rest in the overflow list
+        got = emu_spme(emu, pos, q, (16, 16, 16), p, 0.34, box, cap=cap, repeat=2, tile_log=4)
+        assert got[0] == 0 and ref[0] == 0
+        for a, b in zip(got[1:], ref[1:]):
+            assert np.array_equal(a, b)
+
+
 @pytest.mark.parametrize("K,p,tile_log,pieces", [((32, 40, 48), 4, 3, (5, 7, 8)), ((30, 32, 36), 5, 3, (5, 6, 8)),
                                                  ((32, 40, 48), 6, 4, (3, 4))])
 def test_emulated_k1_pieces_do_not_change_results(emu, oracle_mod, K, p, tile_log, pieces):

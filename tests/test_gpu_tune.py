@@ -69,7 +69,10 @@ def test_every_tiling_candidate_is_bit_identical(pme, oracle_mod, name):
 
 # mesh, order, atoms, the default tile edge on 152 SMs: either side of the tile-count and density lines
 DEFAULT_EDGES = [((80, 80, 96), 6, 5000, 16), ((80, 80, 80), 6, 5000, 8), ((80, 80, 96), 4, 6000, 8), ((72, 80, 100), 4, 6000, 16),
-                 ((80, 80, 96), 8, 4000, 8), ((80, 80, 100), 5, 60000, 16), ((128, 128, 128), 8, 17000, 16)]
+                 ((80, 80, 96), 8, 4000, 8), ((80, 80, 100), 5, 60000, 16), ((128, 128, 128), 8, 17000, 16),
+                 # more atoms in a 16^3 tile than it takes at a time
+                 ((80, 80, 96), 6, 165000, 16), ((72, 80, 100), 8, 245000, 16), ((90, 96, 100), 4, 300000, 8),
+                 ((90, 96, 100), 5, 800000, 16), ((72, 80, 100), 4, 122500, 8)]
 
 
 @pytest.mark.parametrize("K,p,n,edge", DEFAULT_EDGES, ids=[f"{K[0]}x{K[1]}x{K[2]}_p{p}_{n}" for K, p, n, _ in DEFAULT_EDGES])

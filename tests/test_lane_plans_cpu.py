@@ -1,5 +1,6 @@
-"""The register transforms' lane plans and the launch rules that go by them, compiled for the CPU."""
+"""The register transforms' lane plans and the launch rules of the stages, compiled for the CPU."""
 import ctypes
+import math
 import os
 import subprocess
 
@@ -38,3 +39,24 @@ def test_slab_threads_of_groups(lanes, edges):
             assert lanes.lane_slab_threads(K2, K3, 153) == (512 if K2 * K3 <= 10000 else one), (K2, K3)
             assert lanes.lane_slab_threads(K2, K3, 152) == one
     assert lanes.lane_slab_threads(80, 80, 0) > 512 and lanes.lane_slab_threads(108, 108, 1000) > 512
+
+
+@pytest.mark.parametrize("K", [(80, 80, 96), (90, 96, 100), (96, 96, 96), (72, 80, 100), (128, 128, 128), (64, 64, 64)],
+                         ids=lambda K: "x".join(map(str, K)))
+def test_default_tiles_hold_their_atoms(lanes, K):
+    """Atoms beyond a tile's bucket take a path many times slower. At every density and order, buckets of the default
+    16^3 tiles hold at least what the eight 8^3 tiles in each would, and eight times twice the mean over 8^3 tiles
+    (ragged ones among them)."""
+    Kc = (ctypes.c_int * 3)(*K)
+    N = K[0] * K[1] * K[2]
+    for p in (4, 5, 6, 8):
+        edges = set()
+        for density in (0.01, 0.03, 0.06, 0.1, 0.15, 0.2, 0.25, 0.3, 0.4, 0.6, 0.85, 0.95):
+            n = int(density * N)
+            edge = lanes.lane_tile_edge(ctypes.c_longlong(n), Kc, p)
+            cap = lanes.lane_bucket_capacity(ctypes.c_longlong(n), Kc, edge)
+            edges.add(edge)
+            if edge == 16:
+                assert cap >= 8 * lanes.lane_bucket_capacity(ctypes.c_longlong(n), Kc, 8)
+                assert cap >= 16 * n / math.prod((k + 7) // 8 for k in K)
+        assert (16 in edges) == (K != (64, 64, 64)) or p == 4
