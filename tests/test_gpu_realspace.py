@@ -202,11 +202,66 @@ def _water(n, box, seed):
     return (np.random.default_rng(seed).random((n, 3)) @ np.asarray(box)).astype(np.float32), q
 
 
-# atoms, cell, cutoff, what: item and ring edges of the pair kernel, cell and image edges of its neighbourhoods
+def _spread_out(n, box, seed, cluster=1):
+    """n atoms on a jittered lattice of fractional positions, so that no close pair drowns the others; cluster: that many
+    atoms in a row at each site, 2 A apart."""
+    rng = np.random.default_rng(seed)
+    lengths = np.linalg.norm(box, axis=1)
+    m = np.ones(3, int)
+    while m.prod() * cluster < n:
+        m[np.argmax(lengths / m)] += 1
+    cell = np.stack(np.unravel_index(rng.permutation(m.prod()), m), 1)
+    site = ((cell + 0.5 + 0.3 * (rng.random((len(cell), 3)) - 0.5)) / m) @ np.asarray(box)
+    pos = (np.repeat(site, cluster, 0) + 2.0 * np.tile(np.arange(cluster), len(cell))[:, None] * np.array([0.6, 0.0, 0.8]))[:n]
+    return pos.astype(np.float32), rng.normal(size=n).astype(np.float32)
+
+
+def _pair_sums(pos, q, box, beta, rcut):
+    """Real-space forces, energy, virial in FP64 over explicit images, and what FP32 pair terms may be off by: 1e-6 (16
+    roundings) of each term's magnitude, a displacement off by 2 units of the kernel's fixed point (at most 2^-30 of
+    the extent it spans, the largest cell edge or ten cutoffs), and all of a pair within 3e-7 of the cutoff."""
+    from scipy.spatial import cKDTree
+    from scipy.special import erfc
+
+    p, z = pos.astype(np.float64), q.astype(np.float64)
+    inv = np.linalg.inv(box)
+    frac = p @ inv
+    p = (frac - np.floor(frac)) @ box
+    reach = np.ceil(rcut * np.linalg.norm(inv, axis=0)).astype(int)
+    shifts = np.array(np.meshgrid(*[np.arange(-r, r + 1) for r in reach])).reshape(3, -1).T
+    every = (p[None] + (shifts @ box)[:, None]).reshape(-1, 3)
+    owner = np.tile(np.arange(len(p)), len(shifts))
+    near = ((every >= p.min(0) - rcut) & (every <= p.max(0) + rcut)).all(1)
+    every, owner = every[near], owner[near]
+    F, dF, E, dE, V, dV = np.zeros_like(p), np.zeros(len(p)), 0.0, 0.0, np.zeros(6), 0.0
+    u = max(np.abs(box).sum(0).max(), 10.0 * rcut) * 2.0 ** -30
+    tree = cKDTree(every)
+    for c in range(0, len(p), 512):
+        hits = tree.query_ball_point(p[c:c + 512], rcut * (1.0 + 2e-6))
+        i = c + np.repeat(np.arange(len(hits)), [len(h) for h in hits])
+        j = np.concatenate([np.asarray(h, int) for h in hits])
+        d = p[i] - every[j]
+        r = np.sqrt((d * d).sum(1))
+        i, j, d, r = i[r > 0], j[r > 0], d[r > 0], r[r > 0]
+        qq = z[i] * z[owner[j]]
+        e = qq * erfc(beta * r) / r
+        s = (e + qq * 2.0 * beta / np.sqrt(np.pi) * np.exp(-(beta * r) ** 2)) / r ** 2
+        off = np.where(np.abs(r / rcut - 1.0) < 3e-7, 1.0, 1e-6 + 8.0 * u / r)
+        k = r <= rcut
+        np.add.at(F, i[k], s[k, None] * d[k])
+        np.add.at(dF, i, np.abs(s) * r * off)
+        E += 0.5 * e[k].sum()
+        dE += 0.5 * (np.abs(e) * off).sum()
+        V += 0.5 * np.array([(s[k] * d[k, a] * d[k, b]).sum() for a, b in ((0, 0), (1, 1), (2, 2), (0, 1), (0, 2), (1, 2))])
+        dV += 0.5 * (np.abs(s) * r * r * off).sum()
+    return F, E, V, dF, dE, dV
+
+
+# atoms, cell, cutoff (, atoms at a site): item and ring edges of the pair kernel, cell and image edges of its neighbourhoods
 EDGES = {
-    "two_atoms": (2, np.eye(3) * 30.0, 9.0),
+    "two_atoms": (2, np.eye(3) * 12.0, 9.0),
     "one_item": (33, np.eye(3) * 12.0, 5.0),
-    "sparse_rows": (300, np.eye(3) * 120.0, 9.0),          # far fewer atoms than cells
+    "sparse_rows": (300, np.eye(3) * 120.0, 9.0, 5),       # far fewer atoms than cells
     "long_rows": (1500, np.diag([14.0, 15.0, 300.0]), 4.0),  # several slabs per row, coarse fixed point
     "long_other": (1500, np.diag([300.0, 15.0, 14.0]), 4.0),
     "half_cell": (900, np.eye(3) * 20.0, 10.0),            # the cutoff reaches half the cell
@@ -220,27 +275,25 @@ EDGES = {
 
 @pytest.mark.parametrize("name", sorted(EDGES))
 def test_pair_kernel_edges(pme, oracle_mod, name):
-    """Each pair term carries a few FP32 roundings (below 16 of 2^-24, or 1e-6), so the sums stay within 1e-6 of the
-    same sums of magnitudes, which are the oracle's for the absolute charges; the self term is an FP64 sum."""
-    n, box, rcut = EDGES[name]
-    pos, q = _water(n, box, 17)
-    beta = 3.0 / rcut
+    """Every atom's force, the energy and the virial within the sum of what their pair terms may be off by (_pair_sums,
+    itself checked against the oracle). Atoms keep apart and beta rcut = 0.5, so that a pair near the cutoff weighs a
+    hundredth or so of a near one: one pair lost or met twice is hundreds of times the bound."""
+    n, box, rcut = EDGES[name][:3]
+    pos, q = _spread_out(n, box, 17, *EDGES[name][3:])
+    beta = 0.5 / rcut
     er, es, vir, F = gpu_real(pme, pos, q, box, beta, rcut)
+    F0, E, V, dF, dE, dV = _pair_sums(pos, q, box, beta, rcut)
+    assert np.abs(er - E) <= dE
+    assert np.abs(vir - V).max() <= dV
+    assert (np.linalg.norm(F - F0, axis=1) <= dF + 1e-30).all()
     p64, q64 = pos.astype(np.float64), q.astype(np.float64)
     oracle_mod.set_threads(16)
     try:
-        if n > 10000:  # sampled atoms
-            rows = np.random.default_rng(3).choice(n, 60, replace=False)
-            r = oracle_mod.ewald_real_rows(p64, q64, beta, box, rows, rcut=rcut)
-            F = F[rows]
-        else:
-            r = oracle_mod.ewald_real(p64, q64, beta, box, rcut=rcut)
-            big = oracle_mod.ewald_real(p64, np.abs(q64), beta, box, rcut=rcut)
-            assert abs(er - r["energy"]) <= E_REL_TOL * big["energy"]
-            assert np.abs(vir - r["virial"]).max() <= E_REL_TOL * np.abs(big["virial"]).max()
+        rows = np.random.default_rng(3).choice(n, min(n, 60), replace=False)
+        r = oracle_mod.ewald_real_rows(p64, q64, beta, box, rows, rcut=rcut)
     finally:
         oracle_mod.set_threads(1)
-    assert np.abs(F - r["forces"]).max() <= F_RMS_TOL * np.abs(r["forces"]).max()
+    assert np.abs(F0[rows] - r["forces"]).max() <= 1e-10 * np.abs(r["forces"]).max() + dF[rows].max() * 1e-3
     assert es == pytest.approx(oracle_mod.ewald_self(q64, beta), rel=1e-12)
 
 
@@ -296,35 +349,25 @@ def test_gas_costs_no_more_than_liquid(pme):
     assert us[1] < 2.0 * us[0], us
 
 
-# atoms, cell edge, edge of the part of it that they fill: around the line between fine and coarse cells (as many atoms
-# as fine cells, 1000 of them here), and inhomogeneous systems on the coarse side of it
-DENSITIES = {"just_fine": (1000, 50.0, None), "just_coarse": (999, 50.0, None), "gas": (2000, 400.0, None),
-             "droplet": (1500, 120.0, 25.0), "two_droplets": (1500, 300.0, 25.0)}
+# atoms, cell edge, edge of the part of it that they fill, atoms at a site: around the line between fine and coarse cells
+# (as many atoms as fine cells, 1000 of them here), and systems of few atoms a cell
+DENSITIES = {"just_fine": (1000, 50.0, None, 2), "just_coarse": (999, 50.0, None, 2), "gas": (2000, 400.0, None, 4),
+             "droplet": (1500, 120.0, 25.0, 1), "two_droplets": (1500, 300.0, 25.0, 1)}
 
 
 @pytest.mark.parametrize("name", sorted(DENSITIES))
-def test_real_space_at_any_density(pme, oracle_mod, name):
-    """Energy, forces and virial against the oracle for few atoms a cell, both sides of the choice of cells; each within
-    1e-6 of the same sums of magnitudes (16 FP32 roundings a pair term). beta rcut = 0.5 keeps pairs at the cutoff in
-    sight. two_droplets: across two opposite corners of the cell, so that neighbours are images of each other."""
-    n, L, size = DENSITIES[name]
-    rng = np.random.default_rng(41)
-    pos = rng.random((n, 3)) * (L if size is None else size) + (0.0 if size is None else 3.0)
+def test_real_space_at_any_density(pme, name):
+    """Forces, energy and virial within the bounds of _pair_sums (as test_pair_kernel_edges). two_droplets: in two
+    opposite corners of the cell, so that neighbours are images of each other, and half of each a cell further out."""
+    n, L, size, cluster = DENSITIES[name]
+    box = np.eye(3) * L
+    pos, q = _spread_out(n, box if size is None else np.eye(3) * size, 41, cluster)
     if name == "two_droplets":
-        pos[::2] = L - pos[::2] - 1.0
-        pos[:, 0] = np.where(rng.random(n) < 0.5, pos[:, 0], pos[:, 0] - L)
-    pos = pos.astype(np.float32)
-    q = rng.normal(size=n).astype(np.float32)
-    beta = 0.05
-    er, es, vir, F = gpu_real(pme, pos, q, np.eye(3) * L, beta, 10.0)
-    p64, q64 = pos.astype(np.float64), q.astype(np.float64)
-    oracle_mod.set_threads(16)
-    try:
-        r = oracle_mod.ewald_real(p64, q64, beta, np.eye(3) * L, rcut=10.0)
-        big = oracle_mod.ewald_real(p64, np.abs(q64), beta, np.eye(3) * L, rcut=10.0)
-    finally:
-        oracle_mod.set_threads(1)
-    assert abs(er - r["energy"]) <= E_REL_TOL * big["energy"]
-    assert np.abs(vir - r["virial"]).max() <= E_REL_TOL * np.abs(big["virial"]).max()
-    assert np.abs(F - r["forces"]).max() <= F_RMS_TOL * np.abs(r["forces"]).max()
-    assert es == pytest.approx(oracle_mod.ewald_self(q64, beta), rel=1e-12)
+        pos[::2] = (L - 1.0 - pos[::2])
+        pos[::3, 0] -= np.float32(L)
+    er, es, vir, F = gpu_real(pme, pos, q, box, 0.05, 10.0)
+    F0, E, V, dF, dE, dV = _pair_sums(pos, q, box, 0.05, 10.0)
+    assert np.abs(er - E) <= dE
+    assert np.abs(vir - V).max() <= dV
+    assert (np.linalg.norm(F - F0, axis=1) <= dF + 1e-30).all()
+    assert es == pytest.approx(-0.05 / math.sqrt(math.pi) * (q.astype(np.float64) ** 2).sum(), rel=1e-12)
