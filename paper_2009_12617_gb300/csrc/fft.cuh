@@ -223,6 +223,7 @@ PME_DEV void dft_small<10, true>(float2 *v) {
     dft10<true>(v);
 }
 
+#if defined(PME_HOST_EMULATION)
 // Radix chosen for the remaining length rem = N / Ns: 8, then 4, 2, 3, 5.
 PME_DEV int fft_radix(int rem) {
     if (rem % 8 == 0) return 8;
@@ -292,8 +293,10 @@ PME_DEV float2 *fft_batch(float2 *a, float2 *b, int N, int ntr, int es, int bs, 
     }
     return a;
 }
+#endif
 
-#if !defined(PME_HOST_EMULATION)
+// The lane transforms need a warp; PME_EMULATE_WARP says that the including file supplies one on the CPU.
+#if !defined(PME_HOST_EMULATION) || defined(PME_EMULATE_WARP)
 // ---------------------------------------------------------------------------------------------------------
 // Lane-distributed transforms in registers, for lengths N = L * E, L lanes of E points (the lane plans,
 // PME_LANE_CASES). The L lanes of one transform sit in one warp at lane ids t + T j (T = floor(32 / L)
@@ -313,6 +316,27 @@ PME_DEV float2 *fft_batch(float2 *a, float2 *b, int N, int ntr, int es, int bs, 
 // With radices 3 and 5 across lanes, the lengths with those factors need no shared-memory Stockham passes, whose
 // nine barriers and run-time radices bound a slab stage (54 x 60 x 72, one evaluation of 23901 atoms at p = 5:
 // influence stage 19.7 -> 6.3 us, slab stages 18.3 and 18.5 -> 13 us each under ncu, 50.0 -> 33.4 us in all).
+
+// Unit u -> (transform t, lane j): warp u / 32 holds T = floor(32 / L) transforms at lane ids t mod T + T j. Lanes
+// past the last transform get a t beyond any count: they work on a valid transform without storing.
+template <int L>
+PME_DEV void lane_unit(int u, int &t, int &j) {
+    constexpr int T = 32 / L;
+    const int lid = u & 31;
+    t = (u >> 5) * T + (T * L == 32 ? lid & (T - 1) : lid % T);
+    j = lid / T;
+    if (T * L < 32 && j >= L) {
+        t = 1 << 24;
+        j = 0;
+    }
+}
+
+// Units covering ntr transforms of L lanes: whole warps.
+template <int L>
+PME_DEV int lane_units(int ntr) {
+    constexpr int T = 32 / L;
+    return ((ntr + T - 1) / T) * 32;
+}
 
 PME_HD int lane_radix(int M) { return M % 5 == 0 ? 5 : (M % 3 == 0 ? 3 : 2); }
 PME_HD int lane_rounds(int L) { return L <= 1 ? 0 : 1 + lane_rounds(L / lane_radix(L)); }
@@ -518,6 +542,6 @@ PME_DEV void lane_fft_adjoint(float2 (&v)[E], int j, const LaneTw<L, E> &tw) {
     }
     dft_small<E, true>(v);
 }
-#endif  // !PME_HOST_EMULATION
+#endif  // warps
 
 }  // namespace pme

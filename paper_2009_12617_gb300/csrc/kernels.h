@@ -11,6 +11,18 @@
 namespace pme {
 
 constexpr int GB300_SMS = 152;
+
+// The kernels have no other transforms than the lane plans': every accepted mesh has one for each direction.
+constexpr bool every_mesh_has_plans() {
+    for (int i = 0; i < N_EDGES; ++i) {
+        if (conv_lane_plan(mesh_edge(i)) < 0) return false;
+        for (int j = 0; j < N_EDGES; ++j)
+            if (slab_lane_plan(mesh_edge(j) / 2, mesh_edge(i)) < 0 || slab_lane_plan(mesh_edge(i), mesh_edge(j) / 2 + 1) < 0) return false;
+    }
+    return true;
+}
+static_assert(every_mesh_has_plans(), "a mesh edge without lane plans");
+
 constexpr int NT_BIN = 128;    // threads per CTA for binning (BIN_CHUNK atoms per CTA)
 // Threads of the slab CTAs: SLAB_THREADS, or as many more (up to NT_SLAB) as let both passes run in one round of
 // lanes (the plans are chosen to fit SLAB_THREADS where they can; long edges do not). 108^3, whose passes take 704 and

@@ -16,7 +16,8 @@
 #include "common.cuh"
 #include "fft.cuh"
 
-// The register transforms (lane plans) need warps; the CPU emulation keeps only the shared-memory transforms.
+// The register transforms (lane plans) need warps; the CPU emulation, which has one thread per CTA, takes the
+// shared-memory transforms (stage_*_smem, fft_batch), which are built for nothing else.
 #if !defined(PME_HOST_EMULATION)
 #define PME_LANE_FFT 1
 #endif
@@ -143,6 +144,7 @@ inline size_t smem_gather_all(int p, int tlog) {
     return smem_gather(p, tlog) > fin ? smem_gather(p, tlog) : fin;
 }
 
+#if defined(PME_HOST_EMULATION)
 // global -> shared copy of n elements with LOAD_BATCH independent loads in flight per thread
 template <class T>
 PME_DEV void copy_batched(T *dst, const T *src, int n) {
@@ -157,6 +159,7 @@ PME_DEV void copy_batched(T *dst, const T *src, int n) {
             if (base + u * nth < n) dst[base + u * nth] = v[u];
     }
 }
+#endif
 
 // ---------------------------------------------------------------------------------------------------------
 // 64-bit fixed point (scale 2^40) as (hi, lo): rn(v) = hi * 2^20 + lo with lo in [-2^19, 2^19]. The split is
@@ -677,6 +680,7 @@ PME_DEV void stage_spread(const SysDev &d, int item, void *smem, bool cleared = 
 // even/odd pairs plus the split step), then the complex FFT along k2 for every m3 column. (The inverse
 // stage zeroes the slab of the int64 mesh for the next evaluation's spreading.)
 
+#if defined(PME_HOST_EMULATION)
 PME_DEV void stage_fwd_smem(const SysDev &d, int k1, void *smem) {
     const int tid = PME_TID, nth = PME_NTH;
     const int K2 = d.K2, K3 = d.K3, H3 = d.H3, Nh = K3 / 2;
@@ -722,6 +726,7 @@ PME_DEV void stage_fwd_smem(const SysDev &d, int k1, void *smem) {
     float2 *out = d.spec + (size_t)k1 * K2 * H3;
     for (int i = tid; i < K2 * H3; i += nth) out[i] = Y[i];
 }
+#endif
 
 // ---------------------------------------------------------------------------------------------------------
 // a4: pencils (m2, a chunk of m3 columns) — FFT along k1, multiply by the influence function B*C (the
@@ -803,6 +808,7 @@ PME_DEV float2 influence_point(const SysDev &d, int m1, int m2, int m3, int mt2,
     return x;
 }
 
+#if defined(PME_HOST_EMULATION)
 PME_DEV void stage_conv_smem(const SysDev &d, int item, void *smem) {
     const int tid = PME_TID, nth = PME_NTH;
     const int K1 = d.K1, K2 = d.K2, H3 = d.H3;
@@ -869,6 +875,7 @@ PME_DEV void stage_conv_smem(const SysDev &d, int item, void *smem) {
         part[(size_t)item * 8 + c] = s;
     }
 }
+#endif
 
 // ---------------------------------------------------------------------------------------------------------
 // Slab decomposition helpers (the corner turns of the paper's distributed 3D FFT, Sec. III-A "FFT"): copy
@@ -1013,6 +1020,7 @@ PME_DEV void reduce_level2(const SysDev &d, void *smem) {
 // a5: inverse slab k1 — inverse FFT along k2 per m3 column, then the complex-to-real inverse along k3
 // (merge step + a length K3/2 complex FFT whose real / imaginary parts are the even / odd samples).
 
+#if defined(PME_HOST_EMULATION)
 PME_DEV void stage_inv_smem(const SysDev &d, int k1, void *smem) {
     const int tid = PME_TID, nth = PME_NTH;
     const int K2 = d.K2, K3 = d.K3, H3 = d.H3, Nh = K3 / 2;
@@ -1044,6 +1052,7 @@ PME_DEV void stage_inv_smem(const SysDev &d, int k1, void *smem) {
     float2 *out = (float2 *)(d.phi + (size_t)k1 * K2 * K3);  // (phi[2n], phi[2n+1]) = (Re, Im) of R[n]
     for (int i = tid; i < K2 * Nh; i += nth) out[i] = R[i];
 }
+#endif
 
 #if defined(PME_LANE_FFT)
 }  // namespace pme
@@ -1057,27 +1066,6 @@ namespace cg = cooperative_groups;
 // transform directions), the influence stage none before its energy reduction. Thread counts must be
 // multiples of 32; every warp runs whole loop iterations, and lanes past the end work on a valid dummy
 // transform without storing, so the shuffles always see full warps.
-
-// Unit u -> (transform t, lane j): warp u / 32 holds T = floor(32 / L) transforms at lane ids t mod T + T j. Lanes
-// past the last transform get a t beyond any count: they work on a valid transform without storing.
-template <int L>
-PME_DEV void lane_unit(int u, int &t, int &j) {
-    constexpr int T = 32 / L;
-    const int lid = u & 31;
-    t = (u >> 5) * T + (T * L == 32 ? lid & (T - 1) : lid % T);
-    j = lid / T;
-    if (T * L < 32 && j >= L) {
-        t = 1 << 24;
-        j = 0;
-    }
-}
-
-// Units covering ntr transforms of L lanes: whole warps.
-template <int L>
-PME_DEV int lane_units(int ntr) {
-    constexpr int T = 32 / L;
-    return ((ntr + T - 1) / T) * 32;
-}
 
 // Where a slab pass stores its intermediate results: the CTA's own slab buffer and, when a slab is split
 // over a cluster of NB CTAs, the same offset in the other CTAs' buffers (distributed shared memory), so that

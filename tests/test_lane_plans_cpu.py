@@ -4,6 +4,7 @@ import math
 import os
 import subprocess
 
+import numpy as np
 import pytest
 
 from helpers import ROOT
@@ -26,6 +27,36 @@ def lanes():
 def edges(lanes):
     out = (ctypes.c_int * 64)()
     return out[:lanes.lane_edges(out)]
+
+
+def test_lane_transforms(lanes):
+    """Every plan's transforms, by a warp of 32 threads that exchange values as shuffles do: forward and inverse
+    (unnormalised) against a 64-bit FFT, and the adjoint of the forward transform gives N times the input. Each output
+    is a sum of N terms by log2 N levels of a few FP32 roundings: a relative error of 1e-6 in the 2-norm."""
+    for c in range(lanes.lane_plans()):
+        le = (ctypes.c_int * 2)()
+        lanes.lane_plan(c, le)
+        L, E = le
+        N, T = L * E, 32 // L
+        rng = np.random.default_rng(c)
+        x = (rng.normal(size=(T, N)) + 1j * rng.normal(size=(T, N))).astype(np.complex64)
+        out = [np.full((T, N), np.nan, np.complex64) for _ in range(3)]
+        ptr = [a.ctypes.data_as(ctypes.POINTER(ctypes.c_float)) for a in (x, *out)]
+        lanes.lane_run(c, *ptr)
+        x64 = x.astype(np.complex128)
+        for got, ref in zip(out, (np.fft.fft(x64), np.fft.ifft(x64) * N, x64 * N)):
+            assert np.linalg.norm(got - ref) <= 1e-6 * np.linalg.norm(ref), (L, E)
+
+
+def test_stage_shared_memory(lanes, edges):
+    """The slab buffers with their padded rows and the twiddles behind them, and the influence stage's sums, fit the
+    shared memory that the stages are launched with, for every mesh."""
+    used, given = (ctypes.c_longlong * 3)(), (ctypes.c_longlong * 3)()
+    for K2 in edges:
+        for K3 in edges:
+            for K1 in edges if K2 == K3 == 8 else (8,):
+                lanes.lane_smem(K1, K2, K3, used, given)
+                assert all(u <= g for u, g in zip(used, given)), (K1, K2, K3, list(used), list(given))
 
 
 def test_slab_threads_of_groups(lanes, edges):
