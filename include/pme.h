@@ -402,16 +402,15 @@ pme_status pme_batch_sync(pme_batch *batch);
  * waiting (bounded, PME_ETIMEOUT past 1 s) only for its own system's previous stage, so the stages of
  * different systems overlap. PME_BATCH_AUTO (the default): the grouped chains where the systems allow
  * them. Every strategy gives each system its single-system result bit for bit. Takes effect at the next
- * pme_batch_enqueue (which then re-records the graph). Returns PME_EUNSUPPORTED for PME_BATCH_GROUPED
- * when a plan uses 16^3 spreading tiles. Paper: Sec. V-C (several pipelines at once); the work list is
- * this library's own scheduling. */
+ * pme_batch_enqueue (which then re-records the graph). Paper: Sec. V-C (several pipelines at once); the work
+ * list is this library's own scheduling. */
 enum { PME_BATCH_AUTO = 0, PME_BATCH_GROUPED = 1, PME_BATCH_PERSISTENT = 2 };
 pme_status pme_batch_set_strategy(pme_batch *batch, int strategy);
 /* Tune a batch on its own packed DEVICE arrays (as for pme_batch_enqueue): the grouped strategy with every
  * plan's spread / force CTA size at 128, 256 and the density rule, and the persistent strategy, each timed
- * over reps evaluations after a bit-for-bit comparison with the first; the fastest identical one is kept
- * (plans are set to 8^3 tiles, which grouped launches need). *strategy and *us_per_batch (host, either may
- * be NULL) report the choice. Synchronous. */
+ * over reps evaluations after a bit-for-bit comparison with the first; the fastest identical one is kept.
+ * Plans keep their tile edges (the default, or the one set by hand). *strategy and *us_per_batch (host, either
+ * may be NULL) report the choice. Synchronous. */
 pme_status pme_batch_autotune(pme_batch *batch, const float *pos, const float *q, float *forces, double *ev_dev,
                               int reps, int *strategy, double *us_per_batch);
 

@@ -649,7 +649,7 @@ pme_status pme_batch_set_strategy(pme_batch *b, int strategy) {
     if (strategy != PME_BATCH_AUTO && strategy != PME_BATCH_GROUPED && strategy != PME_BATCH_PERSISTENT)
         return fail(PME_EINVAL, "strategy must be PME_BATCH_AUTO, PME_BATCH_GROUPED or PME_BATCH_PERSISTENT");
     if (strategy == PME_BATCH_GROUPED && b->groups.empty())
-        return fail(PME_EUNSUPPORTED, "these systems cannot be grouped (a plan uses 16^3 tiles)");
+        return fail(PME_EUNSUPPORTED, "these systems cannot be grouped");
     b->strategy = strategy;  // the next enqueue re-records the graph if the choice changed
     return PME_OK;
 }
@@ -682,7 +682,7 @@ pme_status pme_batch_autotune(pme_batch *b, const float *pos, const float *q, fl
     pme_status st = PME_OK;
     auto apply = [&](const Cand &c) -> pme_status {
         for (int s = 0; s < nsys; ++s) {
-            pme_status r = plan_retile(b->plans[s], 3, c.nt, b->n[s]);
+            pme_status r = plan_retile(b->plans[s], b->plans[s]->tile_log_set, c.nt, b->n[s]);  // its own edge
             if (r != PME_OK) return r;
         }
         b->strategy = c.strategy;

@@ -190,3 +190,36 @@ def test_batch_autotune_and_refresh(pme):
     finally:
         for pl in plans:
             pme.pme_destroy(pl)
+
+
+@pytest.mark.parametrize("edge", [0, 8], ids=["default", "by_hand"])
+def test_batch_autotune_keeps_tile_edges(pme, edge):
+    """Tuning a batch tries strategies and CTA sizes on its plans' own tile edges: 16 by default at 96^3 (where 8^3 tiles
+    take a quarter longer), or the one set by hand. Results equal the single evaluations bit for bit."""
+    K, n, box = (96, 96, 96), 9000, np.eye(3) * 100.0
+    rng = np.random.default_rng(2)
+    pos = torch.from_numpy((rng.random((2 * n, 3)) * 100.0).astype(np.float32)).cuda()
+    q = torch.from_numpy(rng.normal(size=2 * n).astype(np.float32)).cuda()
+    plans = [pme.pme_create(K, 6, 0.34, box) for _ in range(2)]
+    try:
+        singles = []
+        for i, pl in enumerate(plans):
+            F = torch.empty_like(pos[:n])
+            E, _ = pme.pme_compute(pl, pos[i * n:(i + 1) * n], q[i * n:(i + 1) * n], F)
+            singles.append((E, F))
+            pme.pme_plan_set_tiling(pl, edge, 0)
+        F, ev = torch.empty_like(pos), torch.zeros((2, 7), dtype=torch.float64, device="cuda:0")
+        b = pme.pme_batch_create(plans, [n, n])
+        try:
+            pme.pme_batch_autotune(b, pos, q, F, ev, reps=3)
+            if edge or torch.cuda.get_device_properties(0).multi_processor_count == 152:
+                assert [pme.pme_plan_get_tiling(pl)[0] for pl in plans] == [edge or 16] * 2
+            pme.pme_batch_enqueue(b, pos, q, F, ev)
+            pme.pme_batch_sync(b)
+            for i, (E, Fs) in enumerate(singles):
+                assert ev[i, 0].item() == E and torch.equal(F[i * n:(i + 1) * n], Fs)
+        finally:
+            pme.pme_batch_destroy(b)
+    finally:
+        for pl in plans:
+            pme.pme_destroy(pl)
