@@ -223,8 +223,9 @@ void pme_destroy(pme_plan *plan);
  * anything larger returns PME_EINVAL with the reason. A chain of kernel launches on cuda_stream, then the
  * call waits for them. The first call on a device looks up the array's device address (cudaGetSymbolAddress),
  * loads every kernel a later call may launch and sets a page-locked result block aside, so make that first call
- * before any stream capture. Every call starts by clearing the parts of the array that must be zero, but all calls share the one array: calls that overlap
- * on the GPU (from different streams or threads) race and give wrong results. */
+ * before any stream capture. Every call starts by clearing the parts of the array that must be zero, but all
+ * calls share the one array and the one result block: calls that overlap (from different streams or threads, the
+ * same stream included) race and give wrong results. */
 pme_status pme_compute_noalloc(const int K[3], int p, double beta, const double box[9], const float *pos,
                                const float *q, int64_t n, float *forces, double *energy, double *virial,
                                void *cuda_stream);
@@ -263,7 +264,7 @@ pme_status pme_autotune(pme_plan *plan, const float *pos, const float *q, int64_
 pme_status pme_tune_cache(const char *path);
 
 /* Set the plan's tile edge (0 = default: 16 where the 16^3 tiling has about one tile per SM or more and
- * 32 atoms per tile or more, else 8) and spread / force CTA size (0 = the defaults, chosen per stage by
+ * 32 atoms per tile or more, and at orders 4 and 5 no more than about 1150 in a full tile, else 8) and spread / force CTA size (0 = the defaults, chosen per stage by
  * tile edge and atom density; else 128 or 256, or 512 with tile edge 16, for both stages) by hand; the
  * current configuration is reported by pme_plan_get_tiling (tile_threads 0: the defaults). Batches built on
  * the plan pick the change up at their next pme_batch_enqueue. */

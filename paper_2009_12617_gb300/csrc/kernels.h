@@ -57,8 +57,8 @@ PME_HD int tile_nt_bound(int T) { return T >= 16 ? NT_TILE16 : NT_TILE; }
 // vs 28.75 us per evaluation). 16^3 tiles (hundreds of atoms each) spread on 512 threads. Their force interpolation
 // takes 512 threads too where there are few tiles per SM, so that each ends soon (p = 8, 80 x 80 x 96, 150 tiles: 73 us
 // per evaluation against 88 with 256 or 128 threads); 256 at orders 5 and 6 with few atoms a tile, whose 512 threads
-// would idle (90 x 96 x 100, 25000 atoms, p = 6: 53 against 58 with 512); and 128 where more than three tiles per SM at
-// orders 6 and 8 would come in waves (106 registers at p = 6: four 128-thread CTAs per SM but only one of 512;
+// would idle (90 x 96 x 100, 25000 atoms, p = 6: 53 against 58 with 512); and 128 where more than three tiles per SM (of
+// 152) at orders 6 and 8 would come in waves (106 registers at p = 6: four 128-thread CTAs per SM but only one of 512;
 // 128^3, 262144 atoms, p = 6: 126 against 129 with 256 and 131 with 512). Results do not depend on it.
 inline int tile_threads(const SysDev &d, int64_t n, bool gather = false) {
     if (d.nt_tile == 128 || d.nt_tile == NT_TILE || (d.nt_tile == NT_TILE16 && d.tlog >= 4))
@@ -86,7 +86,8 @@ struct Edge {
 };
 
 // Launch mode of the per-stage kernels: 0 plain, 1 programmatic dependent launch triggered at kernel entry,
-// 2 triggered at CTA exit (see pdl_when for the influence stage), 3 triggered right after the kernel's own wait. Process-wide; affects launches recorded afterwards.
+// 2 triggered at CTA exit (see pdl_when for the influence stage), 3 triggered right after the kernel's own wait.
+// Process-wide; affects launches recorded afterwards.
 void set_launch_mode(int mode);
 int launch_mode();
 // The PdlScope argument of a kernel of stage `stage` of system d in launch mode `mode`. In mode 2 a stage releases

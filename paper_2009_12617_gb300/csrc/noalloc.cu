@@ -7,12 +7,12 @@
 // callers pass only their inputs and outputs; everything else lives in a fixed static device array.
 //
 // How: a set-up kernel clears what must start at zero and writes the mesh's tables, then the six stage kernels of
-// an ordinary evaluation follow on the stream, the last of them storing the result in page-locked host memory. All scratch is
-// carved out of g_noalloc_scratch, a file-scope static __device__ array of NOALLOC_SCRATCH_BYTES that every GPU
+// an ordinary evaluation follow on the stream, the last of them storing the result in page-locked host memory. All
+// scratch is carved out of g_noalloc_scratch, a file-scope static __device__ array of NOALLOC_SCRATCH_BYTES that every GPU
 // loading the library holds until exit. Every kernel a call may need is loaded by the first call on a device
 // (loading one later could take device memory).
 //
-// 2048 atoms, 32^3, p = 4: 52 us a call. One cooperative kernel with nine grid barriers, its table from
+// 2048 atoms, 32^3, p = 4: 52 to 57 us a call. One cooperative kernel with nine grid barriers, its table from
 // a division and two exponentials more per point and its transforms in shared memory took 97 us (88 on the GPU).
 #include <cuda_runtime.h>
 #include <string.h>
@@ -242,7 +242,7 @@ extern "C" pme_status pme_compute_noalloc(const int K[3], int p, double beta, co
     const size_t o_par = off;  off = al256(off + par_bytes);
     const size_t o_grid = off; off = al256(off + K1 * K2 * K3 * 8);
     const size_t zero_bytes = off;
-    off = al256(off + (K1 + K2 + K3) * 8);
+    off = al256(off + (K1 + K2 + K3) * 8);  // unused: the call accepts what it did when B's factors were kept here
     const size_t o_tw = off;   off = al256(off + (K1 + K2 + Nh + Nh + 1) * 8);
     const size_t o_bc = off;   off = al256(off + K1 * K2 * H3 * sizeof(float4));
     const size_t o_spec = off; off = al256(off + K1 * K2 * H3 * 8);

@@ -9,8 +9,7 @@
 // Design. Positions become 32-bit fixed point, modulo 2^32 units u (a power of two chosen so that everything a
 // work item looks at lies within 2^31 units): differences of two atoms are exact integer subtractions, images
 // are integer offsets, and a displacement is rounded once, when it becomes a float. Cells about half a
-// cutoff wide (cells narrower than the cutoff by the factor `sub`, neighbour offsets -R..R) hold the atoms in
-// input-index order, so every sum below runs in an order that depends only on the inputs: results are
+// cutoff wide, or a whole one (real_grid; neighbour offsets -R..R), hold the atoms in input-index order, so every sum below runs in an order that depends only on the inputs: results are
 // bit-reproducible. A work item is up to 32 consecutive sorted atoms of one row of cells (one lane each) and
 // belongs to one CTA, whose warps share out the candidate atoms of the neighbouring rows; see k_rs_pairs. Each
 // pair is visited from both ends, so no atom is written by two CTAs and no force atomics are needed. Energies
@@ -890,8 +889,9 @@ static void rs_launch(void (*kernel)(RealDev), unsigned grid, unsigned block, si
 // sees more of the candidates. Measured with 4 / 8 / 16 warps (us): real space of 2048 atoms 66 / 58 / 54, of 3500
 // - / 50 / 45, of 18000 76 / 82 / -; 32 MD steps of 8190 atoms 2338 / 2019 / 2180, of 12000 1866 / 1692 / -, of 18000
 // 1952 / 2102 / -; full Ewald of 65536 atoms 169 / 193 / 235. (Six warps, three CTAs per SM, for 300 to 456 items: 32
-// steps of 8190 atoms 1424 against 1199 with eight.) A system's sums depend on the number of warps, hence on the atom
-// count alone.
+// steps of 8190 atoms 1424 against 1199 with eight.) All at liquid density: what counts is the number of items, and a
+// gas has more of them for its atoms (2048 atoms at 0.0001 / A^3, 9 A: 62 with 16 warps, 34 with two; 84 with one thread
+// per atom). A system's sums depend on the number of warps, hence on the atom count alone.
 static int rs_pair_warps(const RealDev &d) { return d.n <= 4096 ? 16 : (d.n <= 15000 ? 8 : 4); }
 
 static void launch_pairs(const RealDev &d0, cudaStream_t s) {
