@@ -264,10 +264,11 @@ pme_status pme_autotune(pme_plan *plan, const float *pos, const float *q, int64_
 pme_status pme_tune_cache(const char *path);
 
 /* Set the plan's tile edge (0 = default: 16 where the 16^3 tiling has about one tile per SM or more and
- * 32 atoms per tile or more, and at orders 4 and 5 no more than about 1150 in a full tile, else 8) and spread / force CTA size (0 = the defaults, chosen per stage by
- * tile edge and atom density; else 128 or 256, or 512 with tile edge 16, for both stages) by hand; the
- * current configuration is reported by pme_plan_get_tiling (tile_threads 0: the defaults). Batches built on
- * the plan pick the change up at their next pme_batch_enqueue. */
+ * 32 atoms per tile or more, and at orders 4 and 5 no more than about 1150 in a full tile; else 8) and
+ * spread / force CTA size (0 = the defaults, chosen per stage by tile edge and atom density; else 128 or 256,
+ * or 512 with tile edge 16, for both stages) by hand; the current configuration is reported by
+ * pme_plan_get_tiling (tile_threads 0: the defaults). Batches built on the plan pick the change up at their
+ * next pme_batch_enqueue. */
 pme_status pme_plan_set_tiling(pme_plan *plan, int tile_edge, int tile_threads);
 pme_status pme_plan_get_tiling(const pme_plan *plan, int *tile_edge, int *tile_threads);
 

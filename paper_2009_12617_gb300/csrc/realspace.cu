@@ -9,8 +9,8 @@
 // Design. Positions become 32-bit fixed point, modulo 2^32 units u (a power of two chosen so that everything a
 // work item looks at lies within 2^31 units): differences of two atoms are exact integer subtractions, images
 // are integer offsets, and a displacement is rounded once, when it becomes a float. Cells about half a
-// cutoff wide, or a whole one (real_grid; neighbour offsets -R..R), hold the atoms in input-index order, so every sum below runs in an order that depends only on the inputs: results are
-// bit-reproducible. A work item is up to 32 consecutive sorted atoms of one row of cells (one lane each) and
+// cutoff wide, or a whole one (real_grid; neighbour offsets -R..R), hold the atoms in input-index order, so every sum
+// below runs in an order that depends only on the inputs: results are bit-reproducible. A work item is up to 32 consecutive sorted atoms of one row of cells (one lane each) and
 // belongs to one CTA, whose warps share out the candidate atoms of the neighbouring rows; see k_rs_pairs. Each
 // pair is visited from both ends, so no atom is written by two CTAs and no force atomics are needed. Energies
 // are summed per lane in double-float and across work items in FP64 in a fixed order.
